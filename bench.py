@@ -58,16 +58,19 @@ def mma_flops_per_patch(wl) -> int:
     return wl.K * 2 * up(n) * wl.M * wl.R
 
 
-def kernel_launch_count(slots, K: int, precision: str) -> int:
+REFINE_KERNELS = 1  # kernels of the FP16 path's refine per greedy step and group
+
+
+def kernel_launch_count(slots, K: int, precision: str, refine_kernels: int = 2) -> int:
     """Kernels launched, from the library's per-phase event slots: a scoring
     slot and a hand-off slot are one kernel each; on the FP16 path each group
     has one refine-phase slot around the init kernel and K around the
-    refine's two passes (two kernels each)."""
+    refine's `refine_kernels` kernels."""
     score, handoff, refine = (int(v) for v in slots)
     if precision != "f16":
         return score + handoff + refine
     inits = refine // (K + 1)
-    return score + handoff + inits + 2 * (refine - inits)
+    return score + handoff + inits + refine_kernels * (refine - inits)
 
 
 def algorithmic_bytes_per_patch(wl) -> int:
@@ -984,7 +987,7 @@ def main():
                 "peak_note": ("measured copy bandwidth" if peaks.get("hbm_gbs")
                               else "fallback 6.8 TB/s"),
                 "note": "algorithmic bytes of a launch: read x, write the fp16 residual row; "
-                        "latency-bound (one thread per patch), far below the HBM bound"}
+                        "bound by issue and L1/L2 latency, far below the HBM bound"}
             mf = mma_flops_per_patch(wl)
             mtf = mf * P * args.steps / n_launch / launch_s / 1e12
             line["mma_executed"] = {"flops_per_patch": mf, "tflops": mtf,

@@ -1,6 +1,6 @@
 // romp_refine.cu -- per-patch steps of the FP16 path between scoring passes:
 // candidate certification, exact re-scoring, the least-squares update and the
-// residual (steps (c)-(e) of OMP, Sec. II-C), one thread per patch.
+// residual (steps (c)-(e) of OMP, Sec. II-C).
 //
 // romp_init_kernel writes each patch's packed residual (= x) in fp16 for the
 // first scoring pass and initialises its state.  Rows are scaled by a power
@@ -15,192 +15,206 @@
 //     (disc) is >= s1 - 2E, in which case the patch is handed to the FP32
 //     path;
 //   * re-scores those rows exactly in double-float as
-//     <A_c, x> - sum_i a_i <A_c, A_i> (ties: smallest m*R + r): the slice's
-//     best row first, the others (K <= 5) only when their FP32 score plus its
-//     error bound reaches the exact best;
+//     <A_c, x> - sum_i a_i <A_c, A_i> (ties: smallest m*R + r);
 //   * adds the Cholesky row of the winner (Gram entries and right-hand side
 //     in double-float, factor and solve in FP64) and writes the new residual
 //     row; after the last step the reported residual norm comes from the
 //     factor instead (||x||^2 - z^T z, L z = b).
 // Per-patch state lives in HBM as structure-of-arrays (coalesced over
 // threads); stopped and finished patches write their outputs.
+//
+// One warp works on 32 patches.  What is scalar per patch (candidates, Gram
+// entries, the FP64 factor) runs one thread per patch; what runs over a
+// patch's row (the exact inner product with x, the new residual) runs one
+// warp per row, kBatch rows at a time, its lanes over the row's slots, with
+// the steered atoms read from the dictionary's tables (one 16-byte load per
+// lane and term).  A thread walking its own patch's row and its own atoms'
+// rows instead touches 32 cache lines per warp load; at 10^6 patches of
+// 432 bytes, M = R = 64, K = 5, that kept the L1 tag stage busy for
+// 1.06 ms per step (10,000 cycles per warp and step, DRAM at 16%), while
+// these loads touch the 4 lines of one row.
 #include "rsc_internal.h"
 #include "tc_common.cuh"
 
 namespace {
 
+enum : int { kPlain = 0, kPaired = 1, kLong = 2 };
 
-// State arrays (each of length P, element i of patch p at [field * P + p]).
-template <int KK>
+// State arrays of P patches and K steps (element of patch p at field * P + p).
+// The factor grows by one row per step: L row t (packed lower triangle), its
+// inverse diagonal and z entry are written once, the weights at every step.
 struct StateIdx {
-  static constexpr int nL = KK * (KK + 1) / 2;
-  // doubles: L, inv, z, a
-  static constexpr int dL = 0, dInv = nL, dZ = nL + KK, dA = nL + 2 * KK, nD = nL + 3 * KK;
-  // floats: ahi, alo, xnorm, rnorm, dr, ||x||^2 in double-float (hi, lo)
-  static constexpr int fHi = 0, fLo = KK, fX = 2 * KK, fR = 2 * KK + 1, fDr = 2 * KK + 2,
-                       fX2h = 2 * KK + 3, fX2l = 2 * KK + 4, nF = 2 * KK + 5;
-  // ints: m, r, t, e (exponent of the current row's scale)
-  static constexpr int iM = 0, iR = KK, iT = 2 * KK, iE = 2 * KK + 1, nI = 2 * KK + 2;
+  int dL, dInv, dZ, dA, nD;        // doubles
+  int fHi, fLo, fX, fR, fX2h, fX2l, nF;  // weights in double-float, ||x||, ||r||, ||x||^2
+  int iM, iR, iT, iE, nI;          // atoms, angles, steps of a handed-over patch, row exponent
+  __host__ __device__ explicit StateIdx(int K)
+      : dL(0), dInv(K * (K + 1) / 2), dZ(dInv + K), dA(dZ + K), nD(dA + K),
+        fHi(0), fLo(K), fX(2 * K), fR(2 * K + 1), fX2h(2 * K + 2), fX2l(2 * K + 3), nF(2 * K + 4),
+        iM(0), iR(K), iT(2 * K), iE(2 * K + 1), nI(2 * K + 2) {}
 };
 
-// The selection state (atoms, angles, weights, norms) is loaded when a patch
-// starts; the FP64 factor only right before the Cholesky update, so that it
-// does not hold registers through the scoring code.
-template <int KK>
-__device__ __forceinline__ void load_state(const RefineArgs &a, int64_t p, Ls<KK> &S, int &t,
-                                           int &e, float &xnorm, float &rnorm, float &dr) {
-  using I = StateIdx<KK>;
-  const int64_t P = a.P;
-  t = a.sI[I::iT * P + p];
-  e = a.sI[I::iE * P + p];
+// The slots a lane owns of a packed row: slots 4 lane .. + 3, and for rows of
+// 256 slots 128 + 4 lane .. + 3 too.
+template <int LAY>
+struct LaneSlots {
+  static constexpr int NQ = LAY == kLong ? 2 : 1;
+  int off[4 * NQ];    // float index into the patch's half spectrum, -1: zero slot
+  float wk[4 * NQ];   // weight of the slot in the inner product: 1 (k = 0) or 2
+  unsigned odd;       // slots of odd harmonics
+  bool in;            // the lane's slots are inside the row
+  __device__ LaneSlots(int lane, int J, int kmax) {
+    odd = 0;
+    in = LAY == kLong || 4 * lane < kTcKst;
 #pragma unroll
-  for (int i = 0; i < KK; ++i) {
-    S.ahi[i] = a.sF[(I::fHi + i) * P + p];
-    S.alo[i] = a.sF[(I::fLo + i) * P + p];
-    S.m[i] = a.sI[(I::iM + i) * P + p];
-    S.r[i] = a.sI[(I::iR + i) * P + p];
-  }
-  xnorm = a.sF[I::fX * P + p];
-  rnorm = a.sF[I::fR * P + p];
-  dr = a.sF[I::fDr * P + p];
-}
-
-template <int KK>
-__device__ __forceinline__ void load_factor(const RefineArgs &a, int64_t p, Ls<KK> &S) {
-  using I = StateIdx<KK>;
-  const int64_t P = a.P;
-#pragma unroll
-  for (int q = 0; q < I::nL; ++q) S.L[q] = a.sD[(I::dL + q) * P + p];
-#pragma unroll
-  for (int i = 0; i < KK; ++i) {
-    S.inv[i] = a.sD[(I::dInv + i) * P + p];
-    S.z[i] = a.sD[(I::dZ + i) * P + p];
-    S.a[i] = a.sD[(I::dA + i) * P + p];
-  }
-}
-
-template <int KK>
-__device__ __forceinline__ void store_state(const RefineArgs &a, int64_t p, const Ls<KK> &S, int t,
-                                            int e, float rnorm, float dr) {
-  using I = StateIdx<KK>;
-  const int64_t P = a.P;
-  a.sI[I::iT * P + p] = t;
-  a.sI[I::iE * P + p] = e;
-#pragma unroll
-  for (int q = 0; q < I::nL; ++q) a.sD[(I::dL + q) * P + p] = S.L[q];
-#pragma unroll
-  for (int i = 0; i < KK; ++i) {
-    a.sD[(I::dInv + i) * P + p] = S.inv[i];
-    a.sD[(I::dZ + i) * P + p] = S.z[i];
-    a.sD[(I::dA + i) * P + p] = S.a[i];
-    a.sF[(I::fHi + i) * P + p] = S.ahi[i];
-    a.sF[(I::fLo + i) * P + p] = S.alo[i];
-    a.sI[(I::iM + i) * P + p] = S.m[i];
-    a.sI[(I::iR + i) * P + p] = S.r[i];
-  }
-  a.sF[I::fR * P + p] = rnorm;
-  a.sF[I::fDr * P + p] = dr;
-}
-
-template <int KK>
-__device__ void write_outputs(const RefineArgs &a, int64_t p, const Ls<KK> &S, int t,
-                              float rnorm) {
-  const int K = a.K;
-#pragma unroll
-  for (int i = 0; i < KK; ++i) {
-    if (i < K) {
-      const int64_t o = p * K + i;
-      if (i < t) {
-        a.atom[o] = S.m[i];
-        a.angle_idx[o] = S.r[i];
-        if (a.angle) a.angle[o] = (float)(6.283185307179586 * S.r[i] / a.R);
-        a.coef[o] = S.a[i];
-      } else {
-        a.atom[o] = -1;
-        a.angle_idx[o] = -1;
-        if (a.angle) a.angle[o] = 0.0f;
-        a.coef[o] = 0.0;
-      }
+    for (int u = 0; u < 4 * NQ; ++u) {
+      const int q = (u >> 2) * 128 + 4 * lane + (u & 3);
+      const int code = in ? rsc_slot_code(q, J, kmax, LAY == kPaired) : -1;
+      off[u] = code < 0 ? -1 : 2 * (code >> 8) + (code & 1);
+      const int k = (code >> 1) & 127;
+      wk[u] = code >= 0 && k ? 2.0f : 1.0f;
+      if (code >= 0 && (k & 1)) odd |= 1u << u;
     }
   }
-  if (a.resid_norm2) a.resid_norm2[p] = rnorm * rnorm;
+  __device__ __forceinline__ void load_x(const float *__restrict__ xp, float (&v)[4 * NQ]) const {
+#pragma unroll
+    for (int u = 0; u < 4 * NQ; ++u) v[u] = off[u] >= 0 ? __ldg(xp + off[u]) : 0.0f;
+  }
+  // slots of this lane of table row `row` (rows of L floats)
+  __device__ __forceinline__ void load_row(const float *__restrict__ tab, int row, int lane,
+                                           float (&v)[4 * NQ]) const {
+    constexpr int L = LAY == kLong ? kTcKstLong : kTcKst;
+#pragma unroll
+    for (int q = 0; q < NQ; ++q) {
+      float4 t = make_float4(0.f, 0.f, 0.f, 0.f);
+      if (in) t = __ldg(reinterpret_cast<const float4 *>(tab + (size_t)row * L) + 32 * q + lane);
+      v[4 * q] = t.x;
+      v[4 * q + 1] = t.y;
+      v[4 * q + 2] = t.z;
+      v[4 * q + 3] = t.w;
+    }
+  }
+};
+
+__device__ __forceinline__ df shfl_df(df v, int src) {
+  return {__shfl_sync(0xffffffffu, v.hi, src), __shfl_sync(0xffffffffu, v.lo, src)};
 }
 
-// Shared memory of the init/refine kernels: the steering-factor table
-// [4][H][R], then the packed-slot table qtab[q] = rsc_slot_code (slot q holds
-// Re (c = 0) or Im (c = 1) of entry e = k*J + j, or zero for -1) of the
-// plain or paired row layout.
-__device__ __forceinline__ TwS load_tw(const RefineArgs &a, const int *&qtab) {
-  extern __shared__ __align__(16) float tws[];
-  const int n = 4 * a.H * a.R;
-  for (int i = threadIdx.x; i < n; i += blockDim.x) tws[i] = a.tw[i];
-  int *qt = reinterpret_cast<int *>(tws + ((n + 3) & ~3));
-  for (int q = threadIdx.x; q < a.L; q += blockDim.x)
-    qt[q] = rsc_slot_code(q, a.J, a.kmax, a.paired != 0);
-  __syncthreads();
-  qtab = qt;
-  return TwS{tws, a.H, a.R};
+// Sum kept as a value and the sum of its rounding errors (Dot2, Ogita, Rump,
+// Oishi).
+__device__ __forceinline__ df pair_add(df a, df b) {
+  const df s = two_sum(a.hi, b.hi);
+  return {s.hi, __fadd_rn(s.lo, __fadd_rn(a.lo, b.lo))};
 }
 
-// Packed residual x - sum_i a_i S_{r_i} d_{m_i} of this thread's patch (FP32)
-// written times `scale` as fp16 (L slots, zero-padded) to `row` if not
-// null, slot by slot in packed order; the Im slot of an entry reuses the value
-// computed with its Re slot.  Returns ||r||^2 (unscaled).
-template <int KK>
-__device__ __forceinline__ float residual_q(uint4 *row, int L, float scale,
-                                            const float *__restrict__ xp,
-                                            const float *__restrict__ d, int HJ, int t,
-                                            const Ls<KK> &S, const TwS &tw, const int *qtab) {
-  float n2 = 0.0f, pend = 0.0f;
-#pragma unroll 1
-  for (int cq = 0; cq < L / 8; ++cq) {
-    float v[8];
+// Sums of v[0 .. B) over the lanes (B = 2 or 4): afterwards lane l holds the
+// sum of v[l mod B], over all 32 lanes or (HALF) over its half of the warp.
+// The first log2(B) exchanges halve the values a lane still carries.
+template <int B, bool HALF>
+__device__ __forceinline__ df batch_sum(const df (&v)[B], int lane) {
+  static_assert(B == 2 || B == 4, "batch of two or four rows");
+  df z;
+  if constexpr (B == 4) {
+    df w[2];
 #pragma unroll
-    for (int u = 0; u < 8; ++u) {
-      const int code = qtab[cq * 8 + u];
-      float val = 0.0f;
-      if (code >= 0) {
-        const int e = code >> 8, k = (code >> 1) & 127;
-        if (code & 1) {
-          val = pend;
-        } else {
-          const float2 xv = __ldg(reinterpret_cast<const float2 *>(xp) + e);
-          float re = xv.x, im = k ? xv.y : 0.0f;
+    for (int h = 0; h < 2; ++h) {
+      const df mine = (lane & 1) ? v[2 * h + 1] : v[2 * h];
+      const df give = (lane & 1) ? v[2 * h] : v[2 * h + 1];
+      w[h] = pair_add(mine, df_shfl_xor(give, 1));
+    }
+    const df mine = (lane & 2) ? w[1] : w[0];
+    const df give = (lane & 2) ? w[0] : w[1];
+    z = pair_add(mine, df_shfl_xor(give, 2));
+  } else {
+    const df mine = (lane & 1) ? v[1] : v[0];
+    const df give = (lane & 1) ? v[0] : v[1];
+    z = pair_add(mine, df_shfl_xor(give, 1));
+    z = pair_add(z, df_shfl_xor(z, 2));
+  }
+  z = pair_add(z, df_shfl_xor(z, 4));
+  z = pair_add(z, df_shfl_xor(z, 8));
+  if constexpr (!HALF) z = pair_add(z, df_shfl_xor(z, 16));
+  return z;
+}
+
+template <int B>
+__device__ __forceinline__ float batch_sum_f(const float (&v)[B], int lane) {
+  float z;
+  if constexpr (B == 4) {
+    float w[2];
 #pragma unroll
-          for (int i = 0; i < KK; ++i) {
-            if (i < t) {
-              const float2 dv =
-                  __ldg(reinterpret_cast<const float2 *>(d) + (size_t)S.m[i] * HJ + e);
-              const float dim = k ? dv.y : 0.0f;
-              const float c = tw.cos32(k, S.r[i]), sn = tw.sin32(k, S.r[i]);
-              re = fmaf(-S.ahi[i], fmaf(c, dv.x, sn * dim), re);
-              im = fmaf(-S.ahi[i], fmaf(c, dim, -sn * dv.x), im);
-            }
-          }
-          if (k) {
-            re *= 1.41421356237309515f;
-            pend = im * 1.41421356237309515f;
-          }
-          val = re;
-        }
-        n2 = fmaf(val, val, n2);
-      }
-      v[u] = val;
+    for (int h = 0; h < 2; ++h)
+      w[h] = ((lane & 1) ? v[2 * h + 1] : v[2 * h]) +
+             __shfl_xor_sync(0xffffffffu, (lane & 1) ? v[2 * h] : v[2 * h + 1], 1);
+    z = ((lane & 2) ? w[1] : w[0]) + __shfl_xor_sync(0xffffffffu, (lane & 2) ? w[0] : w[1], 2);
+  } else {
+    z = ((lane & 1) ? v[1] : v[0]) + __shfl_xor_sync(0xffffffffu, (lane & 1) ? v[0] : v[1], 1);
+    z += __shfl_xor_sync(0xffffffffu, z, 2);
+  }
+  z += __shfl_xor_sync(0xffffffffu, z, 4);
+  z += __shfl_xor_sync(0xffffffffu, z, 8);
+  z += __shfl_xor_sync(0xffffffffu, z, 16);
+  return z;
+}
+
+// The next up to B set lanes of `todo` (removed from it); a short batch
+// repeats its first lane.  slot = this lane's place in the batch, or -1.
+template <int B>
+__device__ __forceinline__ void next_batch(unsigned &todo, int lane, int (&src)[B], int &slot) {
+  slot = -1;
+#pragma unroll
+  for (int j = 0; j < B; ++j) {
+    if (todo) {
+      src[j] = __ffs(todo) - 1;
+      todo &= todo - 1;
+      if (lane == src[j]) slot = j;
+    } else {
+      src[j] = src[0];
     }
-    if (row) {
-      uint4 pk;
-      __half2 b0 = __floats2half2_rn(v[0] * scale, v[1] * scale);
-      __half2 b1 = __floats2half2_rn(v[2] * scale, v[3] * scale);
-      __half2 b2 = __floats2half2_rn(v[4] * scale, v[5] * scale);
-      __half2 b3 = __floats2half2_rn(v[6] * scale, v[7] * scale);
-      pk.x = *reinterpret_cast<uint32_t *>(&b0);
-      pk.y = *reinterpret_cast<uint32_t *>(&b1);
-      pk.z = *reinterpret_cast<uint32_t *>(&b2);
-      pk.w = *reinterpret_cast<uint32_t *>(&b3);
-      row[cq] = pk;
+  }
+}
+
+// This lane's slots of a packed row: v (raw entries) times sqrt(2) for k >= 1
+// and `scale`, rounded to fp16; returns the sum of squares of the unscaled
+// packed values.
+template <int LAY>
+__device__ __forceinline__ float store_row(const LaneSlots<LAY> &ls, unsigned char *A, int64_t p,
+                                           int lane, float scale, float (&v)[4 * LaneSlots<LAY>::NQ]) {
+  constexpr int L = LAY == kLong ? kTcKstLong : kTcKst;
+  float n2 = 0.0f;
+#pragma unroll
+  for (int q = 0; q < LaneSlots<LAY>::NQ; ++q) {
+#pragma unroll
+    for (int u = 4 * q; u < 4 * q + 4; ++u) {
+      if (ls.wk[u] == 2.0f) v[u] *= 1.41421356237309515f;
+      n2 = fmaf(v[u], v[u], n2);
     }
+    __half2 b0 = __floats2half2_rn(v[4 * q] * scale, v[4 * q + 1] * scale);
+    __half2 b1 = __floats2half2_rn(v[4 * q + 2] * scale, v[4 * q + 3] * scale);
+    uint2 pk;
+    pk.x = *reinterpret_cast<uint32_t *>(&b0);
+    pk.y = *reinterpret_cast<uint32_t *>(&b1);
+    if (ls.in) reinterpret_cast<uint2 *>(A + p * (int64_t)(2 * L))[32 * q + lane] = pk;
   }
   return n2;
+}
+
+__device__ __forceinline__ void write_none(const RefineArgs &a, int64_t p, int from) {
+  for (int i = from; i < a.K; ++i) {
+    const int64_t o = p * a.K + i;
+    a.atom[o] = -1;
+    a.angle_idx[o] = -1;
+    if (a.angle) a.angle[o] = 0.0f;
+    a.coef[o] = 0.0;
+  }
+}
+
+__device__ __forceinline__ void write_code(const RefineArgs &a, int64_t p, int i, int m, int r,
+                                           double w) {
+  const int64_t o = p * a.K + i;
+  a.atom[o] = m;
+  a.angle_idx[o] = r;
+  if (a.angle) a.angle[o] = (float)(6.283185307179586 * r / a.R);
+  a.coef[o] = w;
 }
 
 // Error bound of one fp16 score of a row of L slots, times 1.25, without the
@@ -226,400 +240,497 @@ __device__ __forceinline__ float score_window(float rnorm, float dr, int e, int 
          ldexpf(1.0f, 16 - e);
 }
 
-template <int KK>
+// Bound on the error of the FP32 residual after t steps with weights whose
+// moduli sum to asum (t = 0: x itself).
+__device__ __forceinline__ float residual_err(int t, float xnorm, float asum) {
+  return t == 0 ? 2.0f * kU32 * xnorm : 2.0f * (t + 6) * kU32 * (xnorm + 1.5f * asum);
+}
+
+template <int LAY>
+struct Batch {  // rows a warp has in flight: registers for B rows of 4 or 8 slots
+  static constexpr int B = LAY == kLong ? 2 : 4;
+};
+
+template <int LAY>
 __global__ void __launch_bounds__(128) romp_init_kernel(const RefineArgs a) {
-  using I = StateIdx<KK>;
-  const int H = a.H, J = a.J, HJ = H * J;
-  const int *qtab;
-  const TwS tw = load_tw(a, qtab);
-  for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < a.P;
-       p += (int64_t)gridDim.x * blockDim.x) {
-    const float *xp = a.x + p * (int64_t)(2 * HJ);
-    df acc = df_make(0.0f);
-    for (int e = 0; e < HJ; ++e) {
-      float2 v = __ldg(reinterpret_cast<const float2 *>(xp) + e);
-      if (e < J) v.y = 0.0f;
-      df q = df_add(two_prod(v.x, v.x), two_prod(v.y, v.y));
-      acc = df_add(acc, e < J ? q : df_mul_f(q, 2.0f));
+  constexpr int NS = 4 * LaneSlots<LAY>::NQ, B = Batch<LAY>::B;
+  const StateIdx I(a.K);
+  const int lane = threadIdx.x & 31, vec = 2 * a.H * a.J;
+  const LaneSlots<LAY> ls(lane, a.J, a.kmax);
+  const int64_t P = a.P, step = (int64_t)gridDim.x * blockDim.x;
+  for (int64_t base = (int64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31); base < P;
+       base += step) {
+    const int64_t p = base + lane;
+    float xnorm = 0.0f, n2 = 0.0f;
+    df x2 = df_make(0.0f);
+    int e = 0;
+    unsigned todo = __ballot_sync(0xffffffffu, p < P);
+    while (todo) {
+      int src[B], slot;
+      next_batch<B>(todo, lane, src, slot);
+      float v[B][NS];
+#pragma unroll
+      for (int j = 0; j < B; ++j) ls.load_x(a.x + (base + src[j]) * vec, v[j]);
+      df s[B];
+#pragma unroll
+      for (int j = 0; j < B; ++j) {
+        s[j] = df_make(0.0f);
+#pragma unroll
+        for (int u = 0; u < NS; ++u) dot2_acc(s[j].hi, s[j].lo, v[j][u], ls.wk[u] * v[j][u]);
+      }
+      df z = batch_sum<B, false>(s, lane);
+      z = fast_two_sum(z.hi, z.lo);  // lane l: the sum of row l mod B
+      const float xn = sqrtf(fmaxf(z.hi + z.lo, 0.0f));
+      const int ez = rsc_row_exponent(xn);
+      float m2[B];
+#pragma unroll
+      for (int j = 0; j < B; ++j) {
+        const int ej = __shfl_sync(0xffffffffu, ez, j);
+        m2[j] = store_row<LAY>(ls, a.A, base + src[j], lane, ldexpf(1.0f, kRowLog2 - ej), v[j]);
+      }
+      const float q2 = batch_sum_f<B>(m2, lane);
+      const int from = slot < 0 ? 0 : slot;
+      const df zx = shfl_df(z, from);
+      const float xr = __shfl_sync(0xffffffffu, xn, from), qr = __shfl_sync(0xffffffffu, q2, from);
+      const int er = __shfl_sync(0xffffffffu, ez, from);
+      if (slot >= 0) {
+        x2 = zx;
+        xnorm = xr;
+        n2 = qr;
+        e = er;
+      }
     }
-    const float xnorm = sqrtf(fmaxf(acc.hi + acc.lo, 0.0f));
-    Ls<KK> S;
-    const int e = rsc_row_exponent(xnorm);
-    const float rn = sqrtf(residual_q<KK>(reinterpret_cast<uint4 *>(a.A + p * (a.L * 2)), a.L,
-                                          ldexpf(1.0f, kRowLog2 - e), xp, a.d, HJ, 0, S, tw,
-                                          qtab));
-    a.sI[I::iT * a.P + p] = 0;
-    a.sI[I::iE * a.P + p] = e;
-    a.sF[I::fX * a.P + p] = xnorm;
-    a.sF[I::fX2h * a.P + p] = acc.hi;
-    a.sF[I::fX2l * a.P + p] = acc.lo;
-    a.sF[I::fR * a.P + p] = rn;
-    a.sF[I::fDr * a.P + p] = 2.0f * kU32 * xnorm;
-    a.win[p] = score_window(rn, 2.0f * kU32 * xnorm, e, a.L);
-    a.status[p] = 1;
+    if (p < P) {
+      const float rn = sqrtf(n2), dr = residual_err(0, xnorm, 0.0f);
+      a.sI[I.iE * P + p] = e;
+      a.sF[I.fX * P + p] = xnorm;
+      a.sF[I.fX2h * P + p] = x2.hi;
+      a.sF[I.fX2l * P + p] = x2.lo;
+      a.sF[I.fR * P + p] = rn;
+      a.win[p] = score_window(rn, dr, e, a.L);
+      a.status[p] = 1;
+    }
   }
 }
 
-// Register budget: 5 blocks of 128 threads per SM (<= 102 registers) up to
-// K = 5; for K = 8 the state (Cholesky row, weights, Gram entries of up to 8
-// atoms) spills 1.8 KB a thread at that budget.  Measured on the 21 x 21-patch
-// image workload: 4 blocks (<= 128 registers, 0.8 KB of spills) 1.9% faster
-// than 3 (<= 168) and 4% faster than 2 (no spills).
+// Step T of every patch still being coded (each has T atoms: a patch that adds
+// none stops), compile-time so that the factor's loops unroll.
 //
-// Two passes per step: a thread re-scores every unit of its patch in one loop,
-// so a warp runs that loop max(units per lane) times.  Nearly all patches have
-// one unit in the window, but among 32 lanes one with several is common, so
-// the first pass (PASS = 1) finishes only the patches with one unit and
-// appends the others to a list, which the second pass (PASS = 2) finishes with
-// every lane on a patch that needs the loop.
-template <int KK, bool PAIRED, int PASS>
-__global__ void __launch_bounds__(128, KK > 5 ? 4 : 5) romp_refine_kernel(const RefineArgs a) {
-  const int H = a.H, J = a.J, R = a.R, M = a.M, HJ = H * J;
-  const int *qtab;
-  const TwS tw = load_tw(a, qtab);
-  const int64_t nwork = PASS == 2 ? (int64_t)*a.slow_count : a.P;
-  for (int64_t w = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; w < nwork;
-       w += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t p = PASS == 2 ? (int64_t)a.slow_list[w] : w;
-    if (a.status[p] <= 0) continue;
-    const float *xp = a.x + p * (int64_t)(2 * HJ);
-    // the patch's row is read by the re-scoring and the residual writer:
-    // start bringing its cache lines into L1 before the state loads
-    // (measured 2.5% on omp_1m)
-    {
-      const uintptr_t b0 = reinterpret_cast<uintptr_t>(xp) & ~(uintptr_t)127;
-      const uintptr_t b1 = reinterpret_cast<uintptr_t>(xp + 2 * HJ - 1);
-      for (uintptr_t q = b0; q <= b1; q += 128) asm volatile("prefetch.global.L1 [%0];" ::"l"(q));
-    }
-    Ls<KK> S;
-    int t, e;
-    float xnorm, rnorm, dr;
-    load_state<KK>(a, p, S, t, e, xnorm, rnorm, dr);
-    // accumulator scores are 2^(16 - e) times the true scores
-    const float unscale = ldexpf(1.0f, e - 16);
-    // the scoring pass's lists of kept blocks (one per column slice of each
-    // chunk, each sorted by block maximum in descending order): their heads
-    // give the best value; the entries are read again by the re-scoring loop
-    // below
-    static_assert(kTcTop == 4, "slots read as float4 / int4 per slice");
-    const float *cvp = a.cand_val + p * kTcCand;
-    const int *cip = a.cand_idx + p * kTcCand;
-    float discm = -INFINITY, head = -INFINITY;
-#pragma unroll
-    for (int sl = 0; sl < kTcSplit; ++sl) {
-      discm = fmaxf(discm, a.cand_disc[kTcSplit * p + sl]);
-      head = fmaxf(head, cvp[kTcTop * sl]);
-    }
-    const float disc = discm * unscale;
-    const float stop_level = 1e-10f * xnorm;
-    const float s1 = head * unscale;
-    // fp16 error of a score (score_err_base) plus a spare 2^-16 s1
-    const float E = score_err_base(rnorm, dr, e, a.L) + 1.52587890625e-5f * fabsf(s1);
+// 10^6 patches, M = R = 64, K = 5: 0.69 ms per step on average (0.62 / 0.81 /
+// 0.98 at T = 1 / 2 / 3) against 1.06 for a thread per patch; the call 9.00 ->
+// 7.29 ms, 1,000 patches at M = 16 261 -> 129 us (one kernel per step, not a
+// memset and two passes), the 21 x 21 image sizes 21.8 -> 16.3 ms.  Issue is
+// at 50%, so both instructions (12,000 to 17,000 per warp) and the loads'
+// latency count.  Registers: at most 128 (4 blocks an SM) 3.79 ms per call of
+// init and refines; without a cap (up to 255) 4.24, 5 or 6 blocks 3.96 / 3.91
+// (spills).
+template <int T, int LAY>
+__global__ void __launch_bounds__(128, 4) romp_refine_kernel(const RefineArgs a) {
+  constexpr int NS = 4 * LaneSlots<LAY>::NQ, B = Batch<LAY>::B;
+  constexpr int TA = T > 0 ? T : 1;
+  constexpr bool PAIRED = LAY == kPaired;
+  constexpr int NP = PAIRED ? 2 : 1;
+  const StateIdx I(a.K);
+  const int lane = threadIdx.x & 31, vec = 2 * a.H * a.J;
+  const int R = a.R, M = a.M, Rr = a.Rr;
+  const LaneSlots<LAY> ls(lane, a.J, a.kmax);
+  const TwS tw{a.tw, a.H, R};  // only for Gram entries without a table
+  const int64_t P = a.P, step = (int64_t)gridDim.x * blockDim.x;
+  for (int64_t base = (int64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31); base < P;
+       base += step) {
+    const int64_t p = base + lane;
+    const bool act = p < P && a.status[p] > 0;
+    if (!__any_sync(0xffffffffu, act)) continue;
+    Ls<T + 1> S;
+    int e = 0;
+    float xnorm = 0.0f, rnorm = 0.0f;
+    float thr = 0.0f, stop_level = 0.0f, unscale = 0.0f;
     int outcome = 0;  // 0 continue, 1 finished/stopped, 2 hand-off
-    bool have_factor = false;
-    if (!(s1 + E > stop_level)) {
-      outcome = 1;
-    } else {
-      const float thr = s1 - 2.0f * E;
-      if (disc >= thr) {
-        outcome = 2;
+    unsigned bmask = 0;
+    int qf = -1, uf = 0;
+    unsigned umk[kTcSplit] = {};
+    if (act) {
+      e = a.sI[I.iE * P + p];
+      xnorm = a.sF[I.fX * P + p];
+      rnorm = a.sF[I.fR * P + p];
+      float asum = 0.0f;
+#pragma unroll
+      for (int i = 0; i < T; ++i) {
+        S.ahi[i] = a.sF[(I.fHi + i) * P + p];
+        S.alo[i] = a.sF[(I.fLo + i) * P + p];
+        S.m[i] = a.sI[(I.iM + i) * P + p];
+        S.r[i] = a.sI[(I.iR + i) * P + p];
+        asum += fabsf(S.ahi[i]);
+      }
+      const float dr = residual_err(T, xnorm, asum);
+      // accumulator scores are 2^(16 - e) times the true scores
+      unscale = ldexpf(1.0f, e - 16);
+      // the scoring pass's lists of kept blocks (one per column slice of each
+      // chunk, each sorted by block maximum in descending order)
+      static_assert(kTcTop == 4, "slots read as float4 / int4 per slice");
+      const float *cvp = a.cand_val + p * kTcCand;
+      const int *cip = a.cand_idx + p * kTcCand;
+      float vv[kTcCand], discm = -INFINITY, head = -INFINITY;
+      int iv[kTcCand];
+      unsigned ubk[kTcSplit];
+#pragma unroll
+      for (int sl = 0; sl < kTcSplit; ++sl) {
+        const float4 v4 = *reinterpret_cast<const float4 *>(cvp + kTcTop * sl);
+        const int4 i4 = *reinterpret_cast<const int4 *>(cip + kTcTop * sl);
+        const uint2 mk = *reinterpret_cast<const uint2 *>(a.cand_mask + 2 * (kTcSplit * p + sl));
+        vv[kTcTop * sl] = v4.x;
+        vv[kTcTop * sl + 1] = v4.y;
+        vv[kTcTop * sl + 2] = v4.z;
+        vv[kTcTop * sl + 3] = v4.w;
+        iv[kTcTop * sl] = i4.x;
+        iv[kTcTop * sl + 1] = i4.y;
+        iv[kTcTop * sl + 2] = i4.z;
+        iv[kTcTop * sl + 3] = i4.w;
+        umk[sl] = mk.x;
+        ubk[sl] = mk.y;
+        discm = fmaxf(discm, a.cand_disc[kTcSplit * p + sl]);
+        head = fmaxf(head, v4.x);
+      }
+      const float disc = discm * unscale, s1 = head * unscale;
+      stop_level = 1e-10f * xnorm;
+      // fp16 error of a score (score_err_base) plus a spare 2^-16 s1
+      const float E = score_err_base(rnorm, dr, e, a.L) + 1.52587890625e-5f * fabsf(s1);
+      if (!(s1 + E > stop_level)) {
+        outcome = 1;
       } else {
-        // a candidate unit is one steered atom (row r*M + m), or in the
-        // paired layout the two angles r and r + R/2 of atom m (row r*M + m,
-        // r < R/2, scored by max(|s(r)|, |s(r + R/2)|)).  Every unit in the
-        // certified window is row b + u of a kept block b (slot q) whose
-        // maximum reaches the window and a column u in its slice's class mask;
-        // the best slice's best unit (the block with the largest maximum and
-        // that slice's best column) is re-scored exactly first.
-        constexpr int NP = PAIRED ? 2 : 1;
-        const int Rh = R / 2;
-        const int MR = PAIRED ? M * Rh : M * R;
-        df best = df_make(0.0f), best_ax = df_make(0.0f);
-        df bg[KK];
-#pragma unroll
-        for (int i = 0; i < KK; ++i) bg[i] = df_make(0.0f);
-        int bm = -1, br = 0, bflat = 0;
-        // the kept blocks inside the window as a bit mask (slot q = slice q / 4);
-        // the loop below runs over (block, column) pairs, so that a warp runs
-        // the re-scoring body max(units per lane) times
-        unsigned bmask = 0;
-        int qf = -1;  // the block with the largest maximum
-        // column mask and best column of slice sl
-        unsigned umk[kTcSplit], ubk[kTcSplit];
-#pragma unroll
-        for (int sl = 0; sl < kTcSplit; ++sl) {
-          const uint2 v = *reinterpret_cast<const uint2 *>(a.cand_mask + 2 * (kTcSplit * p + sl));
-          umk[sl] = v.x;
-          ubk[sl] = v.y;
-        }
-        auto umask_of = [&](int sl) {
-          unsigned r = umk[0];
-#pragma unroll
-          for (int i = 1; i < kTcSplit; ++i) r = sl == i ? umk[i] : r;
-          return r;
-        };
-        auto ubest_of = [&](int sl) {
-          unsigned r = ubk[0];
-#pragma unroll
-          for (int i = 1; i < kTcSplit; ++i) r = sl == i ? ubk[i] : r;
-          return (int)r;
-        };
-        {
+        thr = s1 - 2.0f * E;
+        if (disc >= thr) {
+          outcome = 2;
+        } else {
+          // the kept blocks inside the window as a bit mask (slot q = slice
+          // q / kTcTop); the block with the largest maximum and its slice's
+          // best column come first
           float vbest = -1.0f;
 #pragma unroll
-          for (int sl = 0; sl < kTcSplit; ++sl) {
-            const int4 iq = *reinterpret_cast<const int4 *>(cip + kTcTop * sl);
-            const float4 vq = *reinterpret_cast<const float4 *>(cvp + kTcTop * sl);
-            const int iv[kTcTop] = {iq.x, iq.y, iq.z, iq.w};
-            const float vv[kTcTop] = {vq.x, vq.y, vq.z, vq.w};
-#pragma unroll
-            for (int j = 0; j < kTcTop; ++j)
-              if (iv[j] >= 0 && vv[j] * unscale >= thr) {
-                bmask |= 1u << (sl * kTcTop + j);
-                if (vv[j] > vbest) {
-                  vbest = vv[j];
-                  qf = sl * kTcTop + j;
-                }
-              }
-          }
-        }
-        // (the masks' columns are < 32 by construction; the best column is
-        // masked too, so that candidates left undefined by a scoring pass that
-        // gave up cannot name a row outside the table)
-        const int uf = qf < 0 ? 0 : (ubest_of(qf / kTcTop) & 31);
-        if (PASS == 1) {
-          // units in the window: columns of the masks over the kept blocks
-          int nunits = 0;
-#pragma unroll
           for (int q = 0; q < kTcCand; ++q)
-            if (bmask & (1u << q)) nunits += __popc(umask_of(q / kTcTop));
-          if (nunits > 1) {
-            a.slow_list[atomicAdd(a.slow_count, 1)] = (int)p;
-            continue;
-          }
-        }
-        // The other units are first scored in FP32 and re-scored exactly only
-        // if they can reach the exact best so far.  Error of the FP32 score:
-        // each per-harmonic dot product of J complex entries and the angle
-        // transform over H harmonics round at most 2J + 2H + 8 times, on
-        // terms bounded by ||x|| (unit atoms, Cauchy-Schwarz) and by |a_i| for
-        // the Gram terms, and the weights carry only their hi part; x4 margin.
-        // (only the second pass runs more than one unit; at K = 8 the screen
-        // is built into that pass alone: 2.55 -> 2.18 ms per refine launch on
-        // the 21 x 21 image sizes, where windows hold many units)
-        constexpr bool kScreen = KK <= 5 || PASS == 2;
-        float asum = 0.0f;
-#pragma unroll
-        for (int i = 0; i < KK; ++i)
-          if (i < t) asum += fabsf(S.ahi[i]) + fabsf(S.alo[i]);
-        const float E32 = 4.0f * (float)(2 * J + 2 * H + 8) * kU32 * (xnorm + asum) + asum * kU32;
-        // unit iterator: (q, u) starts at the half's best unit; the rest of
-        // its block's columns, then the other kept blocks' columns follow, so a
-        // lane with one unit runs the body once
-        int q = qf, u = qf < 0 ? 0 : uf;
-        unsigned uleft = qf < 0 ? 0u : (umask_of(qf / kTcTop) & ~(1u << uf));
-        unsigned bleft = qf < 0 ? 0u : (bmask & ~(1u << qf));
-        bool more = qf >= 0, first = true;
-#pragma unroll 1
-        while (more) {
-          const int id = cip[q] + u;
-          bool go = cip[q] >= 0 && cip[q] < MR && id < MR;
-          const int m = id % M, r = id / M;
-          if (PASS != 1 && kScreen && go && !first) {
-            float f;
-            if (PAIRED) {
-              const float2 f2 = score32_pair<KK>(a.d + (size_t)m * HJ * 2, xp, a.xgram, M, J, H,
-                                                 R, m, r, t, S, tw);
-              f = fmaxf(fabsf(f2.x), fabsf(f2.y));
-            } else {
-              f = fabsf(score32<KK>(a.d + (size_t)m * HJ * 2, xp, a.xgram, M, J, H, R, m, r, t, S,
-                                    tw));
-            }
-            // cannot reach (or tie) the best: |best| >= |best.hi| (1 - 2^-22)
-            go = !(f + E32 < fabsf(best.hi) * 0.99999976f);
-          }
-          first = false;
-          if (go) {
-            df ax[NP], sc[NP], gq[NP][KK];
-            if (PAIRED) {
-              const DF2 x2 = score_x_pair(a.d + (size_t)m * HJ * 2, xp, J, H, r, tw);
-              ax[0] = x2.a;
-              ax[NP - 1] = x2.b;
-            } else {
-              ax[0] = score_x(a.d + (size_t)m * HJ * 2, xp, J, H, r, tw);
-            }
-#pragma unroll
-            for (int h = 0; h < NP; ++h) sc[h] = ax[h];
-#pragma unroll
-            for (int i = 0; i < KK; ++i) {
-#pragma unroll
-              for (int h = 0; h < NP; ++h) gq[h][i] = df_make(0.0f);
-              if (i < t) {
-                if (PAIRED) {
-                  const DF2 g2 = gram_entry_pair(a.xgram, M, H, R, m, r, S.m[i], S.r[i], tw);
-                  gq[0][i] = g2.a;
-                  gq[NP - 1][i] = g2.b;
-                } else {
-                  gq[0][i] = gram_entry(a.xgram, M, H, R, m, r, S.m[i], S.r[i], tw);
-                }
-#pragma unroll
-                for (int h = 0; h < NP; ++h)
-                  sc[h] = df_sub(sc[h], df_mul(df{S.ahi[i], S.alo[i]}, gq[h][i]));
+            if (iv[q] >= 0 && vv[q] * unscale >= thr) {
+              bmask |= 1u << q;
+              if (vv[q] > vbest) {
+                vbest = vv[q];
+                qf = q;
               }
             }
+          // (the best column is masked, so that candidates left undefined by
+          // a scoring pass that gave up cannot name a row outside the table)
+          unsigned ub = ubk[0];
 #pragma unroll
-            for (int h = 0; h < NP; ++h) {
-              const int rr = r + h * Rh, flat = m * R + rr;
-              if (bm < 0 || df_abs_gt(sc[h], best) || (df_abs_eq(sc[h], best) && flat < bflat)) {
-                best = sc[h];
-                bm = m;
-                br = rr;
-                bflat = flat;
-                best_ax = ax[h];
+          for (int sl = 1; sl < kTcSplit; ++sl) ub = qf / kTcTop == sl ? ubk[sl] : ub;
+          uf = (int)(ub & 31u);
+        }
+      }
+    }
+    auto umask_of = [&](int sl) {
+      unsigned r = umk[0];
 #pragma unroll
-                for (int i = 0; i < KK; ++i) bg[i] = gq[h][i];
-              }
+      for (int i = 1; i < kTcSplit; ++i) r = sl == i ? umk[i] : r;
+      return r;
+    };
+    // A candidate unit is one steered atom (row r*M + m), or in the paired
+    // layout the two angles r and r + R/2 of atom m (row r*M + m, r < R/2,
+    // scored by max(|s(r)|, |s(r + R/2)|)).  Every unit in the certified
+    // window is row b + u of a kept block b (slot q) whose maximum reaches
+    // the window and a column u in its slice's class mask.  A round of the
+    // loop re-scores one unit of every lane that still has one (c1: 89% of
+    // the patches have one unit, so rounds after the first hold a few lanes).
+    const int Rh = R / 2;
+    const int MR = PAIRED ? M * Rh : M * R;
+    df best = df_make(0.0f), best_ax = df_make(0.0f);
+    df bg[TA];
+#pragma unroll
+    for (int i = 0; i < TA; ++i) bg[i] = df_make(0.0f);
+    int bm = -1, br = 0;
+    int q = qf, u = uf;
+    bool more = qf >= 0;
+    unsigned uleft = more ? (umask_of(qf / kTcTop) & ~(1u << uf)) : 0u;
+    unsigned bleft = more ? (bmask & ~(1u << qf)) : 0u;
+    while (__any_sync(0xffffffffu, more)) {
+      int id = -1;
+      if (more) {
+        const int b0 = a.cand_idx[p * kTcCand + q];
+        if (b0 >= 0 && b0 < MR && b0 + u < MR) id = b0 + u;
+      }
+      const bool go = id >= 0;
+      const int m = go ? id % M : 0, r = go ? id / M : 0;
+      const bool flip = !PAIRED && r >= Rr;
+      const int row = go ? (flip ? id - Rr * M : id) | (flip ? 1 << 30 : 0) : 0;
+      // this unit's Gram entries with the selected atoms (one load each)
+      df gq[NP][TA];
+      if (go) {
+#pragma unroll
+        for (int i = 0; i < T; ++i) {
+          int dr = r - S.r[i];
+          if (dr < 0) dr += R;
+          if (a.gram) {
+            const float2 *gp = a.gram + ((size_t)m * M + S.m[i]) * R;
+            const float2 g0 = __ldg(gp + dr);
+            gq[0][i] = df{g0.x, g0.y};
+            if (PAIRED) {
+              const float2 g1 = __ldg(gp + (dr >= Rh ? dr - Rh : dr + Rh));
+              gq[NP - 1][i] = df{g1.x, g1.y};
             }
-          }
-          if (PASS == 1) break;  // the first pass keeps one-unit patches only
-          // next unit: the next column of this block, else the first column
-          // of the next kept block with a non-empty mask
-          while (uleft == 0 && bleft != 0) {
-            q = __ffs(bleft) - 1;
-            bleft &= bleft - 1;
-            uleft = umask_of(q / kTcTop);
-          }
-          more = uleft != 0;
-          if (more) {
-            u = __ffs(uleft) - 1;
-            uleft &= uleft - 1;
+          } else if (PAIRED) {
+            const DF2 g2 = gram_entry_pair(a.xgram, M, a.H, R, m, r, S.m[i], S.r[i], tw);
+            gq[0][i] = g2.a;
+            gq[NP - 1][i] = g2.b;
+          } else {
+            gq[0][i] = gram_entry(a.xgram, M, a.H, R, m, r, S.m[i], S.r[i], tw);
           }
         }
-        if (bm < 0 || !(fabsf(best.hi) > stop_level)) {
+      }
+      // <A_c, x> in double-float, B rows at a time
+      df axe = df_make(0.0f), axo = df_make(0.0f);
+      unsigned todo = __ballot_sync(0xffffffffu, go);
+      while (todo) {
+        int src[B], slot;
+        next_batch<B>(todo, lane, src, slot);
+        float v[B][NS], h[B][NS];
+        int rw[B];
+#pragma unroll
+        for (int j = 0; j < B; ++j) {
+          rw[j] = __shfl_sync(0xffffffffu, row, src[j]);
+          ls.load_x(a.x + (base + src[j]) * vec, v[j]);
+          ls.load_row(a.rows_hi, rw[j] & ~(1 << 30), lane, h[j]);
+        }
+        df s[B];
+#pragma unroll
+        for (int j = 0; j < B; ++j) {
+          s[j] = df_make(0.0f);
+          float lo[NS];
+          ls.load_row(a.rows_lo, rw[j] & ~(1 << 30), lane, lo);
+#pragma unroll
+          for (int w = 0; w < NS; ++w) {
+            // weight 1 or 2 (exact); odd harmonics change sign with half a turn
+            float xw = ls.wk[w] * v[j][w];
+            if (!PAIRED && (rw[j] >> 30) && ((ls.odd >> w) & 1u)) xw = -xw;
+            dot2_acc(s[j].hi, s[j].lo, h[j][w], xw);
+            s[j].lo = __fmaf_rn(lo[w], xw, s[j].lo);
+          }
+        }
+        // paired rows hold the even harmonics in slots 0 .. 63 (lanes 0 .. 15)
+        // and the odd ones behind them: the two halves of the warp sum E and O
+        const df z = batch_sum<B, PAIRED>(s, lane);
+        const int from = slot < 0 ? 0 : slot;
+        const df ze = shfl_df(z, from);
+        if (slot >= 0) axe = fast_two_sum(ze.hi, ze.lo);
+        if (PAIRED) {
+          const df zo = shfl_df(z, from + 16);
+          if (slot >= 0) axo = fast_two_sum(zo.hi, zo.lo);
+        }
+      }
+      if (go) {
+        df ax[NP];
+        ax[0] = PAIRED ? df_add(axe, axo) : axe;
+        if (PAIRED) ax[NP - 1] = df_sub(axe, axo);
+#pragma unroll
+        for (int h = 0; h < NP; ++h) {
+          df sc = ax[h];
+#pragma unroll
+          for (int i = 0; i < T; ++i) sc = df_sub(sc, df_mul(df{S.ahi[i], S.alo[i]}, gq[h][i]));
+          const int rr = r + h * Rh;
+          if (bm < 0 || df_abs_gt(sc, best) ||
+              (df_abs_eq(sc, best) && m * R + rr < bm * R + br)) {
+            best = sc;
+            bm = m;
+            br = rr;
+            best_ax = ax[h];
+#pragma unroll
+            for (int i = 0; i < T; ++i) bg[i] = gq[h][i];
+          }
+        }
+      }
+      // next unit: the next column of this block, else the first column of
+      // the next kept block with a non-empty mask
+      if (more) {
+        while (uleft == 0 && bleft != 0) {
+          q = __ffs(bleft) - 1;
+          bleft &= bleft - 1;
+          uleft = umask_of(q / kTcTop);
+        }
+        more = uleft != 0;
+        if (more) {
+          u = __ffs(uleft) - 1;
+          uleft &= uleft - 1;
+        }
+      }
+    }
+    bool have_weights = false;
+    int en = 0;
+    float dr1 = 0.0f;
+    if (act && outcome == 0) {
+      if (bm < 0 || !(fabsf(best.hi) > stop_level)) {
+        outcome = 1;
+      } else {
+        double gr[T + 1];
+#pragma unroll
+        for (int i = 0; i < T; ++i) gr[i] = df_to_d(bg[i]);
+        gr[T] = 0.0;
+        // <S_r d_m, S_r d_m> = ||d_m||^2: steering preserves the norm
+        const float2 na = __ldg(a.anorm + bm);
+        const double diag = (double)na.x + (double)na.y;
+        const double rhs = df_to_d(best_ax);
+#pragma unroll
+        for (int i = 0; i < T * (T + 1) / 2; ++i) S.L[i] = a.sD[(I.dL + i) * P + p];
+#pragma unroll
+        for (int i = 0; i < T; ++i) {
+          S.inv[i] = a.sD[(I.dInv + i) * P + p];
+          S.z[i] = a.sD[(I.dZ + i) * P + p];
+        }
+        if (!chol_add<T + 1, T>(S, gr, diag, rhs)) {
           outcome = 1;
         } else {
-          const int mb = bm, rb = br;
-          double gr[KK];
+          have_weights = true;
+          S.m[T] = bm;
+          S.r[T] = br;
+          float asum = 0.0f;
 #pragma unroll
-          for (int i = 0; i < KK; ++i) gr[i] = (i < t) ? df_to_d(bg[i]) : 0.0;
-          // <S_r d_m, S_r d_m> = ||d_m||^2: steering preserves the norm
-          const double diag = (double)a.anorm[mb].x + (double)a.anorm[mb].y;
-          const double rhs = df_to_d(best_ax);
-          load_factor<KK>(a, p, S);
-          have_factor = true;
-          if (!CholAt<KK, 0>::run(t, S, gr, diag, rhs)) {
+          for (int i = 0; i <= T; ++i) asum += fabsf(S.ahi[i]);
+          dr1 = residual_err(T + 1, xnorm, asum);
+          if (T + 1 >= a.K) {
             outcome = 1;
+            // final residual norm from the least-squares solution: with
+            // L z = b (b_i = <A_i, x>, the factor of the Gram of the
+            // selected steered atoms), ||x - sum_i a_i A_i||^2 =
+            // ||x||^2 - z^T z, in FP64 from ||x||^2 in double-float (no
+            // residual is formed: the fp16 row is not needed any more)
+            double zz = 0.0;
+#pragma unroll
+            for (int i = 0; i <= T; ++i) zz = fma(S.z[i], S.z[i], zz);
+            const double x2 = (double)a.sF[I.fX2h * P + p] + (double)a.sF[I.fX2l * P + p];
+            rnorm = (float)sqrt(fmax(x2 - zz, 0.0));
           } else {
+            // the previous residual's norm bounds the new one (least squares
+            // over a larger support)
+            en = rsc_row_exponent(rnorm);
 #pragma unroll
-            for (int i = 0; i < KK; ++i)
-              if (i == t) {
-                S.m[i] = mb;
-                S.r[i] = rb;
-              }
-            ++t;
-            float asum = 0.0f;
-#pragma unroll
-            for (int i = 0; i < KK; ++i)
-              if (i < t) asum += fabsf(S.ahi[i]);
-            dr = 2.0f * (t + 6) * kU32 * (xnorm + 1.5f * asum);
-            if (t >= a.K) {
-              outcome = 1;
-              // final residual norm from the least-squares solution: with
-              // L z = b (b_i = <A_i, x>, the factor of the Gram of the
-              // selected steered atoms), ||x - sum_i a_i A_i||^2 =
-              // ||x||^2 - z^T z, in FP64 from ||x||^2 in double-float (no
-              // residual is formed: the fp16 row is not needed any more)
-              double zz = 0.0;
-#pragma unroll
-              for (int i = 0; i < KK; ++i)
-                if (i < t) zz = fma(S.z[i], S.z[i], zz);
-              const double x2 = (double)a.sF[StateIdx<KK>::fX2h * a.P + p] +
-                                (double)a.sF[StateIdx<KK>::fX2l * a.P + p];
-              rnorm = (float)sqrt(fmax(x2 - zz, 0.0));
-            } else {
-              // the previous residual's norm bounds the new one (least squares
-              // over a larger support)
-              const int en = rsc_row_exponent(rnorm);
-              rnorm = sqrtf(residual_q<KK>(reinterpret_cast<uint4 *>(a.A + p * (a.L * 2)), a.L,
-                                           ldexpf(1.0f, kRowLog2 - en), xp, a.d, HJ, t, S,
-                                           tw, qtab));
-              store_state<KK>(a, p, S, t, en, rnorm, dr);
-              a.win[p] = score_window(rnorm, dr, en, a.L);
+            for (int i = 0; i <= T; ++i) {
+              a.sD[(I.dL + T * (T + 1) / 2 + i) * P + p] = S.L[T * (T + 1) / 2 + i];
+              a.sD[(I.dA + i) * P + p] = S.a[i];
+              a.sF[(I.fHi + i) * P + p] = S.ahi[i];
+              a.sF[(I.fLo + i) * P + p] = S.alo[i];
             }
+            a.sD[(I.dInv + T) * P + p] = S.inv[T];
+            a.sD[(I.dZ + T) * P + p] = S.z[T];
+            a.sI[(I.iM + T) * P + p] = bm;
+            a.sI[(I.iR + T) * P + p] = br;
+            a.sI[I.iE * P + p] = en;
           }
         }
       }
     }
-    if (outcome == 1) {
-      if (!have_factor) {
+    // ---- new residual rows x - sum_i a_i S_{r_i} d_{m_i} (FP32) of the
+    // patches that go on, B rows at a time
+    const bool wr = act && outcome == 0;
+    int rows[T + 1];
 #pragma unroll
-        for (int i = 0; i < KK; ++i)
-          if (i < t) S.a[i] = a.sD[(StateIdx<KK>::dA + i) * a.P + p];
+    for (int i = 0; i <= T; ++i) {
+      const bool flip = wr && S.r[i] >= Rr;
+      rows[i] = wr ? ((flip ? S.r[i] - Rr : S.r[i]) * M + S.m[i]) | (flip ? 1 << 30 : 0) : 0;
+    }
+    unsigned todo = __ballot_sync(0xffffffffu, wr);
+    float rn2 = 0.0f;
+    while (todo) {
+      int src[B], slot;
+      next_batch<B>(todo, lane, src, slot);
+      float v[B][NS];
+#pragma unroll
+      for (int j = 0; j < B; ++j) ls.load_x(a.x + (base + src[j]) * vec, v[j]);
+#pragma unroll
+      for (int i = 0; i <= T; ++i) {
+        float h[B][NS], w[B];
+        int rw[B];
+#pragma unroll
+        for (int j = 0; j < B; ++j) {
+          rw[j] = __shfl_sync(0xffffffffu, rows[i], src[j]);
+          w[j] = __shfl_sync(0xffffffffu, S.ahi[i], src[j]);
+          ls.load_row(a.rows_hi, rw[j] & ~(1 << 30), lane, h[j]);
+        }
+#pragma unroll
+        for (int j = 0; j < B; ++j) {
+          const float wo = (rw[j] >> 30) ? -w[j] : w[j];
+#pragma unroll
+          for (int s = 0; s < NS; ++s)
+            v[j][s] = fmaf(-(((ls.odd >> s) & 1u) ? wo : w[j]), h[j][s], v[j][s]);
+        }
       }
-      write_outputs<KK>(a, p, S, t, rnorm);
+      float m2[B];
+#pragma unroll
+      for (int j = 0; j < B; ++j) {
+        const int ej = __shfl_sync(0xffffffffu, en, src[j]);
+        m2[j] = store_row<LAY>(ls, a.A, base + src[j], lane, ldexpf(1.0f, kRowLog2 - ej), v[j]);
+      }
+      const float z = batch_sum_f<B>(m2, lane);
+      const float zr = __shfl_sync(0xffffffffu, z, slot < 0 ? 0 : slot);
+      if (slot >= 0) rn2 = zr;
+    }
+    if (wr) {
+      const float rn = sqrtf(rn2);
+      a.sF[I.fR * P + p] = rn;
+      a.win[p] = score_window(rn, dr1, en, a.L);
+    } else if (act && outcome == 1) {
+      if (have_weights) {
+#pragma unroll
+        for (int i = 0; i <= T; ++i) write_code(a, p, i, S.m[i], S.r[i], S.a[i]);
+        write_none(a, p, T + 1);
+      } else {
+#pragma unroll
+        for (int i = 0; i < T; ++i)
+          write_code(a, p, i, S.m[i], S.r[i], a.sD[(I.dA + i) * P + p]);
+        write_none(a, p, T);
+      }
+      if (a.resid_norm2) a.resid_norm2[p] = rnorm * rnorm;
       a.status[p] = 0;
-    } else if (outcome == 2) {
-      const int slot = atomicAdd(a.redo_count, 1);
-      a.redo_list[slot] = (int)p;
+    } else if (act) {
+      a.sI[I.iT * P + p] = T;
+      const int at = atomicAdd(a.redo_count, 1);
+      a.redo_list[at] = (int)p;
       if (a.fallbacks) atomicAdd(a.fallbacks, 1ull);
       a.status[p] = -1;
     }
   }
 }
 
-template <int KK>
-int launch_refine_t(const RefineArgs &a, bool init, cudaStream_t stream) {
+template <int LAY>
+int launch_refine_l(const RefineArgs &a, int step, unsigned grid, cudaStream_t stream) {
+  switch (step) {
+    case -1: romp_init_kernel<LAY><<<grid, 128, 0, stream>>>(a); break;
+    case 0: romp_refine_kernel<0, LAY><<<grid, 128, 0, stream>>>(a); break;
+    case 1: romp_refine_kernel<1, LAY><<<grid, 128, 0, stream>>>(a); break;
+    case 2: romp_refine_kernel<2, LAY><<<grid, 128, 0, stream>>>(a); break;
+    case 3: romp_refine_kernel<3, LAY><<<grid, 128, 0, stream>>>(a); break;
+    case 4: romp_refine_kernel<4, LAY><<<grid, 128, 0, stream>>>(a); break;
+    case 5: romp_refine_kernel<5, LAY><<<grid, 128, 0, stream>>>(a); break;
+    case 6: romp_refine_kernel<6, LAY><<<grid, 128, 0, stream>>>(a); break;
+    case 7: romp_refine_kernel<7, LAY><<<grid, 128, 0, stream>>>(a); break;
+    default: return RSC_ERR_UNSUPPORTED;
+  }
+  const cudaError_t e = cudaGetLastError();
+  return e == cudaSuccess ? RSC_OK : rsc_cuda_fail(e);
+}
+
+}  // namespace
+
+void rsc_state_layout(int K, int *nD, int *nF, int *nI) {
+  const StateIdx I(K);
+  *nD = I.nD;
+  *nF = I.nF;
+  *nI = I.nI;
+}
+
+int rsc_launch_refine(const RefineArgs &a, int step, cudaStream_t stream) {
+  if (a.P == 0) return RSC_OK;
   int dev = 0, nsm = 0;
-  cudaError_t e = cudaGetDevice(&dev);
+  const cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return rsc_cuda_fail(e);
   cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
   const int64_t blocks = (a.P + 127) / 128;
   const int64_t cap = (int64_t)nsm * (a.blocks_per_sm > 0 ? a.blocks_per_sm : 32);
   const unsigned grid = (unsigned)(blocks < cap ? blocks : cap);
-  const size_t shm = (size_t)((4 * a.H * a.R + 3) & ~3) * 4 + (size_t)a.L * 4;
-  if (init) {
-    romp_init_kernel<KK><<<grid, 128, shm, stream>>>(a);
-  } else {
-    e = cudaMemsetAsync(a.slow_count, 0, sizeof(int), stream);
-    if (e != cudaSuccess) return rsc_cuda_fail(e);
-    // the second pass's list holds a few percent of the patches: a grid of
-    // 4 blocks per SM walks it
-    const unsigned grid2 = (unsigned)(grid < (unsigned)(nsm * 4) ? grid : (unsigned)(nsm * 4));
-    if (a.paired) {
-      romp_refine_kernel<KK, true, 1><<<grid, 128, shm, stream>>>(a);
-      romp_refine_kernel<KK, true, 2><<<grid2, 128, shm, stream>>>(a);
-    } else {
-      romp_refine_kernel<KK, false, 1><<<grid, 128, shm, stream>>>(a);
-      romp_refine_kernel<KK, false, 2><<<grid2, 128, shm, stream>>>(a);
-    }
-  }
-  e = cudaGetLastError();
-  if (e != cudaSuccess) return rsc_cuda_fail(e);
-  return RSC_OK;
-}
-
-}  // namespace
-
-namespace {
-template <int KK>
-int state_layout_t(int *nD, int *nF, int *nI) {
-  *nD = StateIdx<KK>::nD;
-  *nF = StateIdx<KK>::nF;
-  *nI = StateIdx<KK>::nI;
-  return KK;
-}
-}  // namespace
-
-int rsc_state_layout(int K, int *nD, int *nF, int *nI) {
-  if (K <= 3) return state_layout_t<3>(nD, nF, nI);
-  if (K <= 5) return state_layout_t<5>(nD, nF, nI);
-  return state_layout_t<8>(nD, nF, nI);
-}
-
-int rsc_launch_refine(const RefineArgs &a, bool init, cudaStream_t stream) {
-  if (a.P == 0) return RSC_OK;
-  if (a.K <= 3) return launch_refine_t<3>(a, init, stream);
-  if (a.K <= 5) return launch_refine_t<5>(a, init, stream);
-  if (a.K <= 8) return launch_refine_t<8>(a, init, stream);
-  return RSC_ERR_UNSUPPORTED;
+  if (a.L == kTcKstLong) return launch_refine_l<kLong>(a, step, grid, stream);
+  return a.paired ? launch_refine_l<kPaired>(a, step, grid, stream)
+                  : launch_refine_l<kPlain>(a, step, grid, stream);
 }

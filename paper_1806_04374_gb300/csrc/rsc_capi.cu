@@ -145,6 +145,8 @@ void free_dict(rsc_dict *d) {
   cudaFree(d->paired_f16);
   cudaFree(d->xgram);
   cudaFree(d->anorm);
+  cudaFree(d->rows);
+  cudaFree(d->gram);
   delete d;
 }
 
@@ -237,6 +239,59 @@ __global__ void xgram_kernel(const float *__restrict__ d, int M, int J, int H,
   }
 }
 
+// Steered atoms for the refine: entry q of row r*M + m, r < Rr, is slot q
+// (rsc_slot_code layout) of S_r d_m without the packing weight, FP64 from the
+// double-float steering factors, as a hi plane and a lo plane of rows * L.
+__global__ void refine_rows_kernel(const float *__restrict__ d, const float *__restrict__ tw,
+                                   int M, int J, int kmax, int R, int Rr, int L, int paired,
+                                   float *__restrict__ out) {
+  const int H = kmax + 1, HJ = H * J;
+  const int64_t total = (int64_t)Rr * M * L;
+  for (int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; idx < total;
+       idx += (int64_t)gridDim.x * blockDim.x) {
+    const int q = (int)(idx % L);
+    const int64_t row = idx / L;
+    const int m = (int)(row % M), r = (int)(row / M);
+    const int code = rsc_slot_code(q, J, kmax, paired != 0);
+    float hi = 0.0f, lo = 0.0f;
+    if (code >= 0) {
+      const int e = code >> 8, k = (code >> 1) & 127;
+      const double co = (double)tw[(0 * H + k) * R + r] + (double)tw[(1 * H + k) * R + r];
+      const double si = (double)tw[(2 * H + k) * R + r] + (double)tw[(3 * H + k) * R + r];
+      const double dre = d[((size_t)m * HJ + e) * 2];
+      const double dim = k ? (double)d[((size_t)m * HJ + e) * 2 + 1] : 0.0;
+      const double v = (code & 1) ? co * dim - si * dre : co * dre + si * dim;
+      hi = (float)v;
+      lo = (float)(v - (double)hi);
+    }
+    out[idx] = hi;
+    out[total + idx] = lo;
+  }
+}
+
+// Gram entries of steered atoms, <S_r d_a, d_b> = sum_k w_k Re(e^{ik theta_r}
+// H_k(a, b)) in FP64 from the cross-Gram table, stored as double-float at
+// [(a M + b) R + r].
+__global__ void gram_kernel(const float4 *__restrict__ X, const float *__restrict__ tw, int M,
+                            int H, int R, float2 *__restrict__ G) {
+  const int64_t total = (int64_t)M * M * R;
+  for (int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; idx < total;
+       idx += (int64_t)gridDim.x * blockDim.x) {
+    const int r = (int)(idx % R);
+    const float4 *h = X + (idx / R) * H;
+    double g = 0.0;
+    for (int k = 0; k < H; ++k) {
+      const float4 v = __ldg(h + k);
+      const double co = (double)tw[(0 * H + k) * R + r] + (double)tw[(1 * H + k) * R + r];
+      const double si = (double)tw[(2 * H + k) * R + r] + (double)tw[(3 * H + k) * R + r];
+      const double t = co * ((double)v.x + (double)v.y) - si * ((double)v.z + (double)v.w);
+      g += k ? 2.0 * t : t;
+    }
+    const float hi = (float)g;
+    G[idx] = make_float2(hi, (float)(g - (double)hi));
+  }
+}
+
 // ||d_m||^2 in FP64, stored as double-float.
 __global__ void anorm_kernel(const float *__restrict__ d, int M, int J, int H,
                              float2 *__restrict__ NA) {
@@ -280,6 +335,11 @@ int build_tc_tables(rsc_dict *d, cudaStream_t st) {
   if (e == cudaSuccess && paired) e = cudaMalloc(&d->paired_f16, rows / 2 * kTcKst * 2);
   if (e == cudaSuccess) e = cudaMalloc(&d->xgram, (size_t)M * M * H * sizeof(float4));
   if (e == cudaSuccess) e = cudaMalloc(&d->anorm, (size_t)M * sizeof(float2));
+  d->Rr = R % 2 == 0 ? R / 2 : R;
+  const int64_t nrow = (int64_t)d->Rr * M * L, ng = (int64_t)M * M * R;
+  if (e == cudaSuccess) e = cudaMalloc(&d->rows, (size_t)nrow * 2 * sizeof(float));
+  if (e == cudaSuccess && ng * sizeof(float2) <= kGramMax)
+    e = cudaMalloc(&d->gram, (size_t)ng * sizeof(float2));
   if (e == cudaErrorMemoryAllocation) {
     cudaGetLastError();
     return RSC_ERR_OOM;
@@ -296,6 +356,10 @@ int build_tc_tables(rsc_dict *d, cudaStream_t st) {
   const int64_t nx = (int64_t)M * M * H;
   xgram_kernel<<<(unsigned)((nx + T - 1) / T), T, 0, st>>>(d->d, M, J, H, d->xgram);
   anorm_kernel<<<(M + T - 1) / T, T, 0, st>>>(d->d, M, J, H, d->anorm);
+  refine_rows_kernel<<<(unsigned)((nrow + T - 1) / T), T, 0, st>>>(d->d, d->tw, M, J, d->kmax, R,
+                                                                   d->Rr, L, paired, d->rows);
+  if (d->gram)
+    gram_kernel<<<(unsigned)((ng + T - 1) / T), T, 0, st>>>(d->xgram, d->tw, M, H, R, d->gram);
   e = cudaGetLastError();
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
   if (e != cudaSuccess) return rsc_cuda_fail(e);
@@ -428,7 +492,7 @@ size_t f16_scratch_bytes(int64_t P, int K, int L) {
   return al256((size_t)P * L * 2) + 2 * al256((size_t)P * kTcCand * 4) +
          al256((size_t)P * kTcSplit * 4) + al256((size_t)P * kTcSplit * 8) +
          2 * al256((size_t)P * 4) + al256((size_t)nD * P * 8) + al256((size_t)nF * P * 4) +
-         al256((size_t)nI * P * 4) + 2 * al256((size_t)(P + 4) * 4);
+         al256((size_t)nI * P * 4) + al256((size_t)(P + 4) * 4);
 }
 
 int f16_groups(const rsc_dict *dict, int64_t P, int K, int64_t Pg[], size_t bytes[]) {
@@ -455,7 +519,7 @@ int encode_f16_group(const rsc_dict *dict, const RompArgs &base, unsigned char *
   const int K = base.K;
   if (P == 0) return RSC_OK;
   int nD = 0, nF = 0, nI = 0;
-  const int cap = rsc_state_layout(K, &nD, &nF, &nI);
+  rsc_state_layout(K, &nD, &nF, &nI);
   auto al256 = [](size_t v) { return (v + 255) & ~(size_t)255; };
   unsigned char *q = scratch;
   auto take = [&](size_t b) {
@@ -478,6 +542,10 @@ int encode_f16_group(const rsc_dict *dict, const RompArgs &base, unsigned char *
   ra.xgram = dict->xgram;
   ra.anorm = dict->anorm;
   ra.L = dict->row_len;
+  ra.rows_hi = dict->rows;
+  ra.rows_lo = dict->rows + (size_t)dict->Rr * dict->M * dict->row_len;
+  ra.Rr = dict->Rr;
+  ra.gram = dict->gram;
   ra.A = take((size_t)P * ra.L * 2);
   ra.cand_idx = reinterpret_cast<int *>(take((size_t)P * kTcCand * 4));
   ra.cand_val = reinterpret_cast<float *>(take((size_t)P * kTcCand * 4));
@@ -491,9 +559,6 @@ int encode_f16_group(const rsc_dict *dict, const RompArgs &base, unsigned char *
   int *redo = reinterpret_cast<int *>(take((size_t)(P + 4) * 4));
   ra.redo_count = redo;
   ra.redo_list = redo + 4;
-  int *slow = reinterpret_cast<int *>(take((size_t)(P + 4) * 4));
-  ra.slow_count = slow;
-  ra.slow_list = slow + 4;
   ra.paired = dict->paired_f16 != nullptr ? 1 : 0;
   ra.atom = base.atom;
   ra.angle_idx = base.angle_idx;
@@ -531,7 +596,7 @@ int encode_f16_group(const rsc_dict *dict, const RompArgs &base, unsigned char *
   }
   if (rc == RSC_OK) {
     const int slot = timing_begin(dict, 2, st);
-    rc = rsc_launch_refine(ra, true, st);
+    rc = rsc_launch_refine(ra, -1, st);
     timing_end(dict, slot, st);
   }
   for (int step = 0; step < K && rc == RSC_OK; ++step) {
@@ -540,7 +605,7 @@ int encode_f16_group(const rsc_dict *dict, const RompArgs &base, unsigned char *
     timing_end(dict, slot, st);
     if (rc != RSC_OK) break;
     slot = timing_begin(dict, 2, st);
-    rc = rsc_launch_refine(ra, false, st);
+    rc = rsc_launch_refine(ra, step, st);
     timing_end(dict, slot, st);
   }
   if (rc == RSC_OK) {
@@ -549,7 +614,7 @@ int encode_f16_group(const rsc_dict *dict, const RompArgs &base, unsigned char *
     a.redo_list = ra.redo_list;
     a.resume_sI = ra.sI;
     a.resume_P = P;
-    a.resume_cap = cap;
+    a.resume_cap = K;
     a.fallbacks = nullptr;
     const int slot = timing_begin(dict, 1, st);
     rc = rsc_launch_f32(a, st);

@@ -36,6 +36,13 @@ struct rsc_dict {
   int ke, ko;            // paired: MMA K-steps (16 slots) of the even / odd halves
   float4 *xgram;         // [M][M][H] double-float complex H_k(a,b) = sum_j conj(d_a) d_b
   float2 *anorm;         // [M] ||d_m||^2 in double-float
+  // steered atoms as the refine reads them (romp_refine.cu): rows r*M + m of
+  // row_len FP32 entries, hi plane then lo plane (double-float), without the
+  // packing weights; r < Rr = R/2 for even R (half a turn changes the sign
+  // of the odd harmonics), else R
+  float *rows;
+  int Rr;
+  float2 *gram;          // [M][M][R] double-float <S_r d_a, d_b>; null when over kGramMax bytes
   int n;                 // packed real length J (2 kmax + 1)
   // per-phase timing (diagnostic): event pairs recorded around launches
   int timing;
@@ -66,6 +73,7 @@ constexpr int kTcKstLong = 256;  // row length for packed lengths 113..256 (plai
 constexpr int kTcOdd = 64;   // first slot of the odd harmonics in the paired layout
 constexpr int kTcMaxN = 256; // packed lengths the tensor-core path handles
 constexpr int kTcBN = 128;   // steered atoms per MMA (N) and per TMA box
+constexpr size_t kGramMax = (size_t)1 << 28;  // largest Gram table of the refine (bytes)
 constexpr int kTcMaxK = 8;   // greedy steps the tensor-core path handles
 
 constexpr int kTcSN = 256;   // steered atoms per chunk (MMA N) of the scoring pass
@@ -215,7 +223,8 @@ int rsc_launch_score(const ScoreArgs &a, const CUtensorMap &tmA, const CUtensorM
 int rsc_score_stage_options(int L, int paired, int *dflt, int *other);
 
 // Per-patch steps of the split FP16 path (romp_refine.cu): init (packed x,
-// state) or one refine (certify, re-score, Cholesky, residual).
+// state; step -1) or the refine of greedy step `step` (certify, re-score,
+// Cholesky, residual).
 struct RefineArgs {
   const float *x;
   int64_t P;
@@ -224,6 +233,9 @@ struct RefineArgs {
   const float *tw;       // [4][H][R]
   const float4 *xgram;
   const float2 *anorm;   // [M] ||d_m||^2 in double-float
+  const float *rows_hi, *rows_lo;  // see rsc_dict::rows
+  int Rr;
+  const float2 *gram;    // see rsc_dict::gram (null: entries from xgram)
   unsigned char *A;      // [P][L] fp16 packed residual rows, scaled (see below)
   int L;                 // packed row length (kTcKst or kTcKstLong)
   const int *cand_idx;
@@ -243,17 +255,12 @@ struct RefineArgs {
   float *resid_norm2;
   int *redo_list;
   int *redo_count;
-  // [P] + counter: patches whose window holds more than one unit, finished by
-  // the refine's second pass (see romp_refine.cu)
-  int *slow_list;
-  int *slow_count;
   unsigned long long *fallbacks;
   int blocks_per_sm;  // grid cap of the init/refine launches per SM (0: 32)
 };
-int rsc_launch_refine(const RefineArgs &a, bool init, cudaStream_t stream);
-// Number of double / float / int state arrays for K steps; returns the
-// compile-time capacity used (K rounded up to 3, 5 or 8).
-int rsc_state_layout(int K, int *nD, int *nF, int *nI);
+int rsc_launch_refine(const RefineArgs &a, int step, cudaStream_t stream);
+// Number of double / float / int state arrays for K steps.
+void rsc_state_layout(int K, int *nD, int *nF, int *nI);
 
 struct RompArgs {
   const float *x;
