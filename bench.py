@@ -950,7 +950,7 @@ def main():
                               "host buffers, H2D of x and D2H of every output inside); median "
                               "call"},
             "gpu_launches": kernel_launch_count(main_run["kernel_launches"], wl.K,
-                                                args.precision),
+                                                args.precision, REFINE_KERNELS),
             "handoffs": main_run["handoffs"],
             "kernel_ms_per_step": {"scoring": main_run["kernel_ms"][0] / args.steps,
                                    "fp32_handoff": main_run["kernel_ms"][1] / args.steps,
