@@ -53,7 +53,9 @@ struct rsc_basis {
   int KPw, sbw;
   CUtensorMap tmW;
   int *err;      // device error word of the projection kernels (bounded waits)
-  float *Xs;     // device [n][npix]: real synthesis matrix (packed columns), FP32
+  // synthesis matrix for rsc_synthesize (see rsc_basis_view)
+  float *Xs;
+  int ldx, syn_cols;
 };
 
 namespace {
@@ -943,7 +945,19 @@ int rsc_basis_create(int32_t N, int32_t J, int32_t kmax, double ring_width, doub
   if (e == cudaSuccess && tc_ok) e = cudaMalloc(&b->Bt, Bt.size() * sizeof(uint16_t));
   if (e == cudaSuccess && tc_ok)
     e = cudaMemcpy(b->Bt, Bt.data(), Bt.size() * sizeof(uint16_t), cudaMemcpyHostToDevice);
-  std::vector<float> Xf(X.begin(), X.end());  // [n][npix] (column-major X)
+  // synthesis rows by half-spectrum coordinate: Re c[j, 0] at 2 j (its Im has
+  // a zero row), sqrt2 times the packed columns for k >= 1 (pixel = sum over
+  // packed columns of X times sqrt2 c)
+  {
+    const int tiles = (npix + 127) / 128;
+    b->syn_cols = ((npix + tiles - 1) / tiles + 7) / 8 * 8;
+    b->ldx = tiles * b->syn_cols;
+  }
+  std::vector<float> Xf((size_t)(nout + kSynPad) * b->ldx, 0.0f);
+  for (int q = 0; q < n; ++q)
+    for (int p = 0; p < npix; ++p)
+      Xf[(size_t)(q < J ? 2 * q : J + q) * b->ldx + p] =
+          (float)(X[(size_t)q * npix + p] * (q < J ? 1.0 : M_SQRT2));
   if (e == cudaSuccess) e = cudaMalloc(&b->Xs, Xf.size() * sizeof(float));
   if (e == cudaSuccess)
     e = cudaMemcpy(b->Xs, Xf.data(), Xf.size() * sizeof(float), cudaMemcpyHostToDevice);
@@ -1166,6 +1180,6 @@ int rsc_images_scratch_bytes(const rsc_basis *b, int64_t P, int32_t n_images, ui
 
 int rsc_basis_internals(const rsc_basis *b, rsc_basis_view *v) {
   if (!b || !v) return RSC_ERR_INVALID;
-  *v = rsc_basis_view{b->device, b->npix, b->n, b->J, b->nout, b->Xs};
+  *v = rsc_basis_view{b->device, b->npix, b->n, b->J, b->nout, b->Xs, b->ldx, b->syn_cols};
   return RSC_OK;
 }

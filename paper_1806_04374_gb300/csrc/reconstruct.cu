@@ -6,9 +6,9 @@
 //   (steering of Eq. (Sr): harmonic k of an atom times exp(-i k 2 pi r / R)),
 //   accumulated to about 48 bits from the dictionary's FP32 atoms and its
 //   double-float steering factors, rounded once to FP32.
-// rsc_synthesize: pixels = Phi x_hat over the circular patch, one thread per
-//   (patch, pixel), with the basis's real synthesis matrix (FP32, [n][npix],
-//   columns in the packed order: Re of k = 0, then sqrt2 Re and sqrt2 Im).
+// rsc_synthesize: pixels = Phi x_hat over the circular patch, a tiled FP32
+//   matrix product with the basis's real synthesis matrix (rows in the half
+//   spectrum's order, the packing weights folded in).
 #include <algorithm>
 
 #include "df.cuh"
@@ -252,30 +252,184 @@ cudaError_t launch_reconstruct(const rsc_dict *dict, int dev, int64_t P, int K, 
   return cudaGetLastError();
 }
 
-__global__ void synthesize_kernel(const float *__restrict__ X, int n, int npix, int J, int64_t P,
-                                  const float *__restrict__ coef, int nout,
-                                  float *__restrict__ pix) {
-  const int64_t total = P * npix;
-  for (int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; idx < total;
-       idx += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t p = idx / npix;
-    const int q = (int)(idx - p * npix);
-    const float *c = coef + p * nout;
-    float acc = 0.0f;
-    // packed coefficient of column col: Re c[k=0][col] for col < J, else
-    // sqrt2 times half-spectrum entry J + col (Re or Im of c[j][k >= 1])
-    for (int col = 0; col < J; ++col) acc = fmaf(X[(int64_t)col * npix + q], c[2 * col], acc);
-    for (int col = J; col < n; ++col)
-      acc = fmaf(X[(int64_t)col * npix + q], 1.41421356237309515f * c[J + col], acc);
-    pix[idx] = acc;
+// ------------------------------------------------------------- synthesize
+//
+// C[P][npix] = coef[P][nk] X[nk][npix], FP32 FMA in the order of the half
+// spectrum (the error of the plain sum; the tensor cores' accumulation is
+// coarser).  A block takes 16 RT rows and up to 128 pixels; thread (tx, ty)
+// of ct x 16 holds RT x 8 outputs.  Both operands stream through shared memory in chunks of kc coordinates with
+// cp.async, two chunks in flight.  ct, the threads across the pixels, is
+// chosen so that the last tile of pixels is full (97 pixels: 13 x 8 = 104).
+// The result leaves through shared memory, so that its rows are written with
+// full lines.
+// 10^6 patches of 102 coordinates to 97 pixels: 0.68 ms (issue at 65%: seven
+// warps share four schedulers), against 4.0 ms for one output per thread (an X
+// and a coefficient load for every FMA); the FP32 floor is 0.25, the memory
+// floor 0.12.  Two-element FMAs took 0.80 ms (each takes 2.3 cycles on this
+// part), lanes along the pixels instead of the rows 0.80 (13 groups of pixels
+// meet banks twice).
+constexpr int kSynK = kSynPad;  // longest chunk (coordinates)
+constexpr int kSynRows = 16;    // threads down the rows
+
+// A chunk of coefficients is kept transposed, [k][16 RT rows]; groups of four
+// rows are permuted by k so that the transposing copies meet no bank twice.
+__device__ __forceinline__ int syn_a_group(int kq, int group) {
+  return group ^ (kq & 7);
+}
+
+__device__ __forceinline__ void cp_async4(uint32_t dst, const float *src, bool in) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(dst), "l"(src), "r"(in ? 4 : 0)
+               : "memory");
+}
+__device__ __forceinline__ void cp_async16(uint32_t dst, const float *src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
+}
+
+template <int RT>
+__global__ void __launch_bounds__(256, RT == 8 ? 2 : 4)
+    synthesize_kernel(const float *__restrict__ X, int nk, int ldx, int npix, int J, int kc,
+                      int64_t P, const float *__restrict__ coef, int ct, int ntn, bool vec,
+                      float *__restrict__ pix) {
+  constexpr int BM = kSynRows * RT;
+  extern __shared__ __align__(16) float syn_smem[];
+  const int BN = 8 * ct, nthr = kSynRows * ct;
+  const int stage = kc * (BM + BN), kq4 = kc / 4, inv = 65536 / kq4 + 1;
+  const uint32_t s0 = static_cast<uint32_t>(__cvta_generic_to_shared(syn_smem));
+  // rows vary fastest over the lanes: a warp reads 16 different row groups and
+  // two pixel groups, which meets no bank twice
+  const int tid = threadIdx.x, ty = tid % kSynRows, tx = tid / kSynRows;
+  const int64_t ntiles = (P + BM - 1) / BM * ntn;
+  const int nchunk = (nk + kc - 1) / kc;
+  for (int64_t t = blockIdx.x; t < ntiles; t += gridDim.x) {
+    const int64_t p0 = t / ntn * BM;
+    const int n0 = (int)(t % ntn) * BN, nn = min(BN, npix - n0);
+    const int rows = (int)min((int64_t)BM, P - p0);
+    const float *cp0 = coef + p0 * nk;
+    auto load = [&](int c) {
+      const uint32_t sa = s0 + (uint32_t)((c & 1) * stage) * 4, sx = sa + kc * BM * 4;
+      const int k0 = c * kc;
+      // coefficients: kc / 4 threads along a row's chunk, 4 values each
+      for (int i = tid; i < BM * kq4; i += nthr) {
+        const int row = (i * inv) >> 16, kq = i - row * kq4, g = k0 + 4 * kq;  // i < 2^11
+        const uint32_t dst =
+            sa + 16 * (kq * BM + syn_a_group(kq, row >> 2)) + 4 * (row & 3);
+        const float *src = cp0 + row * nk + g;
+        if (row < rows && g >= 2 * J && g + 4 <= nk) {
+#pragma unroll
+          for (int u = 0; u < 4; ++u) cp_async4(dst + 4 * BM * u, src + u, true);
+        } else {
+          // rows past the end, coordinates past nk and the imaginary parts of
+          // k = 0 read as zero
+#pragma unroll
+          for (int u = 0; u < 4; ++u) {
+            const bool in = row < rows && g + u < nk && !(g + u < 2 * J && (u & 1));
+            cp_async4(dst + 4 * BM * u, in ? src + u : coef, in);
+          }
+        }
+      }
+      // X is padded with zeros to whole tiles of BN columns and by kSynK rows
+      const float *xs = X + (size_t)k0 * ldx + n0;
+      for (int i = tid; i < kc * 2 * ct; i += nthr) {
+        const int k = i / (2 * ct), q = i - k * 2 * ct;
+        cp_async16(sx + 4 * (k * BN + 4 * q), xs + (size_t)k * ldx + 4 * q);
+      }
+      asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    float acc[RT][8];
+#pragma unroll
+    for (int i = 0; i < RT; ++i)
+#pragma unroll
+      for (int j = 0; j < 8; ++j) acc[i][j] = 0.0f;
+    load(0);
+    for (int c = 0; c < nchunk; ++c) {
+      if (c + 1 < nchunk) {
+        load(c + 1);
+        asm volatile("cp.async.wait_group 1;" ::: "memory");
+      } else {
+        asm volatile("cp.async.wait_group 0;" ::: "memory");
+      }
+      __syncthreads();
+      const float *sa = syn_smem + (c & 1) * stage, *sx = sa + kc * BM + 8 * tx;
+#pragma unroll 1
+      for (int kq = 0; kq < kq4; ++kq, sa += 4 * BM, sx += 4 * BN) {
+        const float *g0, *g1 = nullptr;
+        if constexpr (RT == 8) {
+          g0 = sa + 4 * syn_a_group(kq, ty);
+          g1 = sa + 4 * syn_a_group(kq, 16 + ty);
+        } else {
+          g0 = sa + 4 * syn_a_group(kq, ty >> 1) + 2 * (ty & 1);
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          float a[RT], b[8];
+          if constexpr (RT == 8) {
+            const float4 a0 = *reinterpret_cast<const float4 *>(g0 + u * BM);
+            const float4 a1 = *reinterpret_cast<const float4 *>(g1 + u * BM);
+            a[0] = a0.x; a[1] = a0.y; a[2] = a0.z; a[3] = a0.w;
+            a[4] = a1.x; a[5] = a1.y; a[6] = a1.z; a[7] = a1.w;
+          } else {
+            const float2 a0 = *reinterpret_cast<const float2 *>(g0 + u * BM);
+            a[0] = a0.x; a[1] = a0.y;
+          }
+          const float4 b0 = *reinterpret_cast<const float4 *>(sx + u * BN);
+          const float4 b1 = *reinterpret_cast<const float4 *>(sx + u * BN + 4);
+          b[0] = b0.x; b[1] = b0.y; b[2] = b0.z; b[3] = b0.w;
+          b[4] = b1.x; b[5] = b1.y; b[6] = b1.z; b[7] = b1.w;
+#pragma unroll
+          for (int i = 0; i < RT; ++i)
+#pragma unroll
+            for (int j = 0; j < 8; ++j) acc[i][j] = fmaf(a[i], b[j], acc[i][j]);
+        }
+      }
+      __syncthreads();
+    }
+    // ---- out through shared memory: the tile's rows of nn pixels, packed
+#pragma unroll
+    for (int i = 0; i < RT; ++i) {
+      const int row = RT == 8 ? (i < 4 ? 4 * ty + i : 60 + 4 * ty + i) : 2 * ty + i;
+#pragma unroll
+      for (int j = 0; j < 8; ++j)
+        if (8 * tx + j < nn) syn_smem[row * nn + 8 * tx + j] = acc[i][j];
+    }
+    __syncthreads();
+    if (ntn == 1) {  // whole rows: the tile is one contiguous piece
+      float *o = pix + p0 * npix;
+      const int total = rows * npix, quads = vec ? total / 4 : 0;
+      for (int i = tid; i < quads; i += nthr)
+        reinterpret_cast<float4 *>(o)[i] = reinterpret_cast<const float4 *>(syn_smem)[i];
+      for (int i = 4 * quads + tid; i < total; i += nthr) o[i] = syn_smem[i];
+    } else {
+      const int lane = tid & 31, w = tid >> 5, nw = nthr >> 5;
+      for (int r = w; r < rows && w < nw; r += nw)
+        for (int j = lane; j < nn; j += 32) pix[(p0 + r) * npix + n0 + j] = syn_smem[r * nn + j];
+    }
+    __syncthreads();
   }
 }
 
-unsigned grid_for(int64_t total, int device) {
-  int nsm = 0;
-  cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, device);
-  const int64_t blocks = (total + 255) / 256, cap = (int64_t)nsm * 16;
-  return (unsigned)(blocks < cap ? blocks : cap);
+template <int RT>
+cudaError_t launch_synthesize(const rsc_basis_view &v, int dev, int64_t P, const float *coef,
+                              float *pixels, cudaStream_t st) {
+  constexpr int BM = kSynRows * RT;
+  const int ct = v.syn_cols / 8, ntn = (v.npix + v.syn_cols - 1) / v.syn_cols;
+  // chunk length: the one that pads the coordinates least
+  int kc = kSynK;
+  for (int c = kSynK - 4; c >= 24; c -= 4)
+    if ((v.nout + c - 1) / c * c < (v.nout + kc - 1) / kc * kc) kc = c;
+  const size_t smem = std::max((size_t)2 * kc * (BM + 8 * ct), (size_t)BM * 8 * ct) * 4;
+  auto kern = synthesize_kernel<RT>;
+  cudaError_t e =
+      cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  int nsm = 0, per_sm = 0;
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+  if (e == cudaSuccess)
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kSynRows * ct, smem);
+  if (e != cudaSuccess) return e;
+  const int64_t tiles = (P + BM - 1) / BM * ntn, cap = (int64_t)nsm * std::max(per_sm, 1);
+  const bool vec = (reinterpret_cast<uintptr_t>(pixels) & 15) == 0;
+  kern<<<(unsigned)std::min(tiles, cap), kSynRows * ct, smem, st>>>(
+      v.X, v.nout, v.ldx, v.npix, v.J, kc, P, coef, ct, ntn, vec, pixels);
+  return cudaGetLastError();
 }
 
 }  // namespace
@@ -314,9 +468,11 @@ extern "C" int rsc_synthesize(const rsc_basis *basis, const float *coef, int64_t
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return rsc_cuda_fail(e);
   if (dev != v.device) return RSC_ERR_INVALID;
-  const int64_t total = P * v.npix;
-  synthesize_kernel<<<grid_for(total, dev), 256, 0, reinterpret_cast<cudaStream_t>(stream)>>>(
-      v.X, v.n, v.npix, v.J, P, coef, v.nout, pixels);
-  e = cudaGetLastError();
+  int nsm = 0;
+  cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+  cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
+  // tiles of 128 patches when they fill the SMs, else of 32
+  e = (P + 127) / 128 >= nsm ? launch_synthesize<8>(v, dev, P, coef, pixels, st)
+                             : launch_synthesize<2>(v, dev, P, coef, pixels, st);
   return e == cudaSuccess ? RSC_OK : rsc_cuda_fail(e);
 }

@@ -167,9 +167,14 @@ int rsc_launch_tc(const TcArgs &a, const CUtensorMap &tmap, cudaStream_t stream)
 int rsc_encode_rows_map(CUtensorMap *map, void *base, size_t rows, int box_rows, int row_len);
 
 // What other translation units need of a basis handle (basis.cu owns it).
+constexpr int kSynPad = 40;  // >= the chunks rsc_synthesize reads
 struct rsc_basis_view {
   int device, npix, n, J, nout;
-  const float *X;  // device [n][npix]: real synthesis matrix, packed column order
+  // device: synthesis matrix by half-spectrum coordinate (nout rows and
+  // kSynPad rows of zeros, of ldx floats: whole tiles of syn_cols pixels), the
+  // weight of the negative harmonics folded in
+  const float *X;
+  int ldx, syn_cols;
 };
 int rsc_basis_internals(const rsc_basis *basis, rsc_basis_view *view);
 // Scratch bytes rsc_encode_images takes for its work list and projected

@@ -1,12 +1,13 @@
 """The way back at the edges of its kernels: rsc_reconstruct's two layouts
 (16-byte pieces or single entries), its longest codes, missing steps, weights
-outside the range of its FP32 accumulator and entries that cancel."""
+outside the range of its FP32 accumulator and entries that cancel;
+rsc_synthesize's tiles of 128 and 32 patches and of up to 128 pixels."""
 import ctypes
 
 import numpy as np
 import pytest
 
-from oracle import ksvd
+from oracle import basis as obasis, ksvd
 from paper_1806_04374_gb300 import synth
 
 pytestmark = pytest.mark.gpu
@@ -87,3 +88,30 @@ def test_reconstruct_weights_out_of_range_and_cancelling(rsc):
     assert np.all(got[3] == 0.0)
     assert np.isnan(got[5][1:]).all() and not np.isfinite(got[4][1:]).any()
     assert np.isinf(got[6][1:]).all()
+
+
+@pytest.mark.parametrize("shape", [
+    # (N, J, kmax, P): four pixels; tiles of 104 pixels; three tiles; partial
+    # tiles of 32 and of 128 patches
+    (2, 1, 0, 3), (3, 1, 1, 40), (11, 6, 8, 1), (11, 6, 8, 33), (11, 6, 8, 19457 + 128),
+    (13, 5, 6, 129), (21, 10, 12, 65), (21, 10, 12, 20000)], ids=str)
+def test_synthesize_edges(rsc, shape):
+    """n FP32 multiply-adds per pixel: within n 2^-24 sum |X c| (and the
+    rounding of X), the imaginary parts of k = 0 ignored."""
+    import torch
+    N, J, kmax, P = shape
+    rng = np.random.default_rng(P)
+    c = rng.standard_normal((P, kmax + 1, J, 2)).astype(np.float32)
+    c[:, 0, :, 1] = np.nan
+    b = rsc.Basis(N, J, kmax)
+    got = rsc.synthesize(b, torch.from_numpy(c).cuda()).cpu().numpy()
+    b.close()
+    c[:, 0, :, 1] = 0.0
+    idx = np.unique(np.r_[np.arange(min(P, 64)), np.arange(max(0, P - 160), P)])
+    ref = obasis.synthesize(c[idx], N, J, kmax)
+    X = np.stack([obasis.synthesize(e, N, J, kmax)[0] for e in
+                  np.eye(c[0].size).reshape(-1, 1, kmax + 1, J, 2)])
+    X[1:2 * J:2] = 0.0
+    bound = np.abs(c[idx].reshape(len(idx), -1)).astype(np.float64) @ np.abs(X)
+    n = J * (2 * kmax + 1)
+    assert np.all(np.abs(got[idx] - ref) <= (n + 4) * 2.0 ** -24 * bound + 1e-30)
