@@ -277,35 +277,146 @@ __global__ void __launch_bounds__(128) project_kernel(const ImageItem *items, in
 // FP32 accumulator: about 2^-21 relative, FP32 accuracy for the coder.  Each
 // window's pixels are scaled by a power of two 2^sa with max |x| 2^sa in
 // [2^13, 2^14) and the operator by 2^sb, far from fp16's range limits; the
-// result is multiplied back by 2^-(sa + sb) (exact).  Two groups of 128
-// threads per CTA each own a tile, an A area and 128 TMEM columns; a group
-// gathers its windows into 128-byte-swizzled K-major rows, one thread issues
-// the 3 x KP/16 MMAs (M = 128, N = NP) and commits them to the group's
-// mbarrier (bounded wait), and every thread reads its window's row back with
-// tcgen05.ld and writes the half spectrum.
-constexpr int kPjThreads = 256;
+// result is multiplied back by 2^-(sa + sb) (exact).
+//
+// Bound by issue (pixel loads, conversions) and by how well the phases of a
+// tile overlap; the output, 4 nout bytes a window, is the memory floor (0.26
+// ms for 4.15 M windows of 11 x 11).  Two groups of 256 threads per CTA each
+// own a tile, an A area and 128 TMEM columns, so that one group's MMAs and
+// copies run beside the other's conversions.  Two threads per window read its
+// pixels once into registers (offsets from a table in shared memory), agree on
+// its scale, and write hi and lo into 128-byte-swizzled K-major rows; one
+// thread issues the 3 x KP/16 MMAs (M = 128, N = NP) and commits them to the
+// group's mbarrier (bounded wait); the next tile's pixels are read while they
+// run; then the group reads its accumulator back into the A area, which is
+// free by then, and one bulk copy takes the tile, a contiguous piece of the
+// output, to memory.  4.15 M windows of 11 x 11: 1.50 -> 0.60 ms against one
+// thread per window that read its pixels twice and wrote its row itself.
+// Slower: an epilogue of its own warps (0.67 ms, they become the bound), one
+// pipeline of 512 threads over all tiles (0.90), the next tile's pixels
+// consumed after the epilogue (0.67).
+constexpr int kPjGroup = 256;  // threads of a group: two per window
+constexpr int kPjThreads = 2 * kPjGroup;
 constexpr int kPjRows = 128;
-constexpr int kPjBlkA = kPjRows * 128;  // one 64-pixel block of a 128-window tile
+constexpr int kPjBlkA = kPjRows * 128;     // one 64-pixel block of a 128-window tile
+constexpr int kPjAreaA = 2 * 2 * kPjBlkA;  // hi, lo; two blocks each
 constexpr uint64_t kPjWaitNs = 2000000000ull;
 
 struct PjLayout {
-  int b_off, a_off, bar_off, total;
+  int b_off, a_off, off_off, max_off, bar_off, total;
 };
 __host__ __device__ inline PjLayout pj_layout(int NP) {
-  const int bblk = NP * 128;                   // one 64-pixel block of the operator
-  const int b_bytes = 2 * 2 * bblk;            // hi, lo; two blocks each
-  const int a_bytes = 2 * 2 * 2 * kPjBlkA;     // two groups; hi, lo; two blocks
-  return PjLayout{0, b_bytes, b_bytes + a_bytes, b_bytes + a_bytes + 64 + 1024};
+  const int a = 2 * 2 * NP * 128;    // operator: hi, lo; two 64-pixel blocks each
+  const int off = a + 2 * kPjAreaA;  // two groups: pixel offsets
+  const int mx = off + 2 * 128 * 4;  // each thread's largest pixel
+  const int bar = mx + kPjThreads * 4;
+  return PjLayout{0, a, off, mx, bar, bar + 64 + 1024};
 }
 
 __device__ __forceinline__ void group_sync(int g) {
-  asm volatile("bar.sync %0, %1;" ::"r"(g + 1), "r"(kPjRows) : "memory");
+  asm volatile("bar.sync %0, %1;" ::"r"(g + 1), "n"(kPjGroup) : "memory");
 }
 
+// The image of flat window p: the last item with first <= p.
+__device__ __forceinline__ int find_item(const ImageItem *items, int n_items, int64_t p) {
+  int lo = 0, hi = n_items - 1;
+  while (lo < hi) {
+    const int mid = (lo + hi + 1) >> 1;
+    if (items[mid].first <= p) lo = mid; else hi = mid - 1;
+  }
+  return lo;
+}
+
+// Top-left pixel of window p (null past the end) and its image's width.
+// `one`: the whole tile p0 .. last lies in one image (the same answer for
+// every thread of the tile).
+__device__ __forceinline__ const float *find_window(const ImageItem *items, int n_items, int N,
+                                                    int64_t p0, int64_t last, int64_t p, int &w,
+                                                    bool &one) {
+  int it = find_item(items, n_items, p0);
+  one = it == n_items - 1 || items[it + 1].first > last;
+  if (p > last) p = last;
+  if (!one) it = find_item(items, n_items, p);
+  const ImageItem im = items[it];
+  const int64_t local = p - im.first;
+  const int nw = im.w - N + 1;
+  int r0, c0;
+  if (local <= 0xffffffffll) {
+    r0 = (int)((uint32_t)local / (uint32_t)nw);
+    c0 = (int)((uint32_t)local - (uint32_t)r0 * (uint32_t)nw);
+  } else {
+    r0 = (int)(local / nw);
+    c0 = (int)(local - (int64_t)r0 * nw);
+  }
+  w = im.w;
+  return im.img + (int64_t)r0 * im.w + c0;
+}
+
+// Offsets of a window's pixels: from the group's table (a tile inside one
+// image) or from the mask and the thread's own image width.  Pixels past npix
+// read the mask's first one.
+struct PixelOffsets {
+  const int *tab;
+  const int2 *offs;
+  int w, npix;
+  bool one;
+  template <int V>
+  __device__ __forceinline__ void load(const float *base, int q, float (&v)[V]) const {
+    if (one) {
+#pragma unroll
+      for (int u = 0; u < V; u += 4) {
+        const int4 o = *reinterpret_cast<const int4 *>(tab + q + u);
+        v[u] = __ldg(base + o.x);
+        v[u + 1] = __ldg(base + o.y);
+        v[u + 2] = __ldg(base + o.z);
+        v[u + 3] = __ldg(base + o.w);
+      }
+    } else {
+#pragma unroll
+      for (int u = 0; u < V; ++u) {
+        const int2 o = __ldg(offs + (q + u < npix ? q + u : 0));
+        v[u] = __ldg(base + (int64_t)o.x * w + o.y);
+      }
+    }
+  }
+};
+
+// Eight pixels times `scale` as fp16 hi and lo parts (EDGE: zeros past npix).
+template <bool EDGE>
+__device__ __forceinline__ void split8(const float (&v)[8], int q, int npix, float scale, uint4 &hi,
+                                       uint4 &lo) {
+  uint32_t hv[4], lv[4];
+#pragma unroll
+  for (int u = 0; u < 4; ++u) {
+    float x0 = v[2 * u] * scale, x1 = v[2 * u + 1] * scale;
+    if (EDGE && q + 8 > npix) {
+      if (q + 2 * u >= npix) x0 = 0.0f;
+      if (q + 2 * u + 1 >= npix) x1 = 0.0f;
+    }
+    const __half2 hh = __floats2half2_rn(x0, x1);
+    const float2 hf = __half22float2(hh);
+    const __half2 ll = __floats2half2_rn(x0 - hf.x, x1 - hf.y);
+    hv[u] = *reinterpret_cast<const uint32_t *>(&hh);
+    lv[u] = *reinterpret_cast<const uint32_t *>(&ll);
+  }
+  hi = make_uint4(hv[0], hv[1], hv[2], hv[3]);
+  lo = make_uint4(lv[0], lv[1], lv[2], lv[3]);
+}
+
+// The power of two that takes a window's largest pixel below 2^14.
+__device__ __forceinline__ int pixel_scale(float amax) {
+  int ea = 0;
+  (void)frexpf(amax, &ea);
+  return 14 - (ea < -100 ? -100 : (ea > 127 ? 127 : ea));
+}
+
+// NC: 8-pixel chunks of a thread (half of KP = 16 NC padded pixels).
+template <int NC>
 __global__ void __launch_bounds__(kPjThreads, 1)
     project_tc_kernel(const ImageItem *items, int n_items, int64_t P_total, int N, int npix,
-                      const int2 *offs, const uint16_t *Bt, int KP, int NP, int sb, int nout,
-                      float *coef, int *err) {
+                      const int2 *offs, const uint16_t *Bt, int NP, int sb, int nout, float *coef,
+                      int *err) {
+  constexpr int KP = 16 * NC, kchunks = 2 * NC;
   extern __shared__ unsigned char pj_raw[];
   unsigned char *smem = reinterpret_cast<unsigned char *>(
       (reinterpret_cast<uintptr_t>(pj_raw) + 1023) & ~uintptr_t(1023));
@@ -315,8 +426,8 @@ __global__ void __launch_bounds__(kPjThreads, 1)
   uint64_t *bars = reinterpret_cast<uint64_t *>(smem + Lo.bar_off);
   uint32_t *s_tmem = reinterpret_cast<uint32_t *>(bars + 2);
   volatile int *s_ok = reinterpret_cast<volatile int *>(bars + 2) + 1;  // [2]
-  const int tid = threadIdx.x, warp = tid >> 5, g = tid >> 7, row = tid & 127;
-  const int kchunks = KP / 8;  // 16-byte chunks of a row
+  const int tid = threadIdx.x, warp = tid >> 5, g = tid / kPjGroup, gt = tid % kPjGroup;
+  const int row = gt & 127, half = gt >> 7;
 
   // operator hi / lo -> swizzled K-major tiles (row = output, 8 pixels a chunk)
   for (int i = tid; i < 2 * NP * kchunks; i += kPjThreads) {
@@ -338,75 +449,72 @@ __global__ void __launch_bounds__(kPjThreads, 1)
   tc::fence_after_sync();
   const uint32_t tmem = *s_tmem;
   const uint32_t bar = tc::smem_u32(bars + g);
-  unsigned char *sA = smem + Lo.a_off + g * (2 * 2 * kPjBlkA);  // hi blocks, then lo blocks
+  unsigned char *sA = smem + Lo.a_off + g * kPjAreaA;  // hi blocks, then lo blocks
   const uint32_t a_hi = tc::smem_u32(sA), a_lo = a_hi + 2 * kPjBlkA;
   const uint32_t b_hi = tc::smem_u32(sB), b_lo = b_hi + 2 * bblk;
   const uint32_t idesc = tc::idesc_f16_f32(kPjRows, NP);
   const uint32_t dcol = tmem + (uint32_t)(g * kPjRows);
   const uint32_t lane_base = (uint32_t)((warp & 3) * 32) << 16;
-  const int64_t ntiles = (P_total + kPjRows - 1) / kPjRows;
+  const int64_t ntiles = (P_total + kPjRows - 1) / kPjRows, step = (int64_t)gridDim.x * 2;
+  int *s_off = reinterpret_cast<int *>(smem + Lo.off_off) + g * 128;
+  float *s_max = reinterpret_cast<float *>(smem + Lo.max_off) + g * kPjGroup;
+  PixelOffsets px{s_off, offs, 0, npix, false};
+  int tab_w = -1;
+  float v[NC][8];
+  // finds this thread's window of tile t, reads its half of the pixels and
+  // hands over their largest
+  auto begin = [&](int64_t t) {
+    const int64_t p0 = t * kPjRows, last = min(p0 + kPjRows, P_total) - 1;
+    const float *base = find_window(items, n_items, N, p0, last, p0 + row, px.w, px.one);
+    if (px.one && px.w != tab_w) {  // the same for the whole group
+      group_sync(g);                // the previous table is read
+      if (gt < KP) {
+        const int2 o = __ldg(offs + (gt < npix ? gt : 0));
+        s_off[gt] = o.x * px.w + o.y;
+      }
+      tab_w = px.w;
+      group_sync(g);
+    }
+#pragma unroll
+    for (int c = 0; c < NC; ++c) px.load<8>(base, 8 * (half * NC + c), v[c]);
+    float amax = 0.0f;
+#pragma unroll
+    for (int c = 0; c < NC; ++c)
+#pragma unroll
+      for (int u = 0; u < 8; ++u) amax = fmaxf(amax, fabsf(v[c][u]));
+    s_max[gt] = amax;
+  };
   uint32_t iter = 0;
   bool alive = true;
-  for (int64_t t = (int64_t)blockIdx.x * 2 + g; t < ntiles && alive;
-       t += (int64_t)gridDim.x * 2, ++iter) {
-    // ---- gather this thread's window, scale, split, write its A rows
-    const int64_t p = t * kPjRows + row;
-    const float *base = nullptr;
-    int w = 0;
-    float amax = 0.0f;
-    if (p < P_total) {
-      int lo = 0, hi = n_items - 1;  // last item with first <= p
-      while (lo < hi) {
-        const int mid = (lo + hi + 1) >> 1;
-        if (items[mid].first <= p) lo = mid; else hi = mid - 1;
-      }
-      const ImageItem it = items[lo];
-      const int64_t local = p - it.first;
-      const int nw = it.w - N + 1;
-      const int r0 = (int)(local / nw), c0 = (int)(local - (int64_t)r0 * nw);
-      base = it.img + (int64_t)r0 * it.w + c0;
-      w = it.w;
-      for (int q = 0; q < npix; ++q) {
-        const int2 o = __ldg(offs + q);
-        amax = fmaxf(amax, fabsf(__ldg(base + (int64_t)o.x * w + o.y)));
-      }
-    }
-    int ea = 0;
-    (void)frexpf(amax, &ea);
-    const int sa = 14 - (ea < -100 ? -100 : (ea > 127 ? 127 : ea));  // max |x| 2^sa < 2^14
-    const float scale = ldexpf(1.0f, sa);
-    for (int c = 0; c < kchunks; ++c) {
-      uint32_t hv[4], lv[4];
+  int64_t t = (int64_t)blockIdx.x * 2 + g;
+  if (t < ntiles) begin(t);
+  for (; t < ntiles && alive; t += step, ++iter) {
+    // ---- scale, split and write this thread's part of its A row (the area
+    // holds the previous tile's outputs until their copy has read them)
+    if (iter > 0 && gt == 0) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
+    group_sync(g);
+    const int sa = pixel_scale(fmaxf(s_max[row], s_max[row + 128]));
+    const float scale = __int_as_float((sa + 127) << 23);  // 2^sa, |sa| < 126
 #pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        float x2[2];
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-          const int q = c * 8 + 2 * u + h;
-          float x = 0.0f;
-          if (base && q < npix) {
-            const int2 o = __ldg(offs + q);
-            x = __ldg(base + (int64_t)o.x * w + o.y) * scale;
-          }
-          x2[h] = x;
-        }
-        const __half2 hh = __floats2half2_rn(x2[0], x2[1]);
-        const float2 hf = __half22float2(hh);
-        const __half2 ll = __floats2half2_rn(x2[0] - hf.x, x2[1] - hf.y);
-        hv[u] = *reinterpret_cast<const uint32_t *>(&hh);
-        lv[u] = *reinterpret_cast<const uint32_t *>(&ll);
-      }
+    for (int i = 0; i < NC; ++i) {
+      const int c = half * NC + i;
+      uint4 hi, lo;
+      // KP - 16 < npix: only the last two chunks reach past the pixels
+      if (i < NC - 2)
+        split8<false>(v[i], c * 8, npix, scale, hi, lo);
+      else
+        split8<true>(v[i], c * 8, npix, scale, hi, lo);
       const int off = (c >> 3) * kPjBlkA + row * 128 + (((c & 7) ^ (row & 7)) << 4);
-      *reinterpret_cast<uint4 *>(sA + off) = make_uint4(hv[0], hv[1], hv[2], hv[3]);
-      *reinterpret_cast<uint4 *>(sA + 2 * kPjBlkA + off) = make_uint4(lv[0], lv[1], lv[2], lv[3]);
+      *reinterpret_cast<uint4 *>(sA + off) = hi;
+      *reinterpret_cast<uint4 *>(sA + 2 * kPjBlkA + off) = lo;
     }
     tc::fence_proxy_async_smem();
     tc::fence_before_sync();
     group_sync(g);
     tc::fence_after_sync();
     // ---- MMAs: hi*hi + hi*lo + lo*hi into the group's accumulator
-    if (row == 0) {
-      const int ks_n = KP / 16;
+    if (gt == 0) {
+      constexpr int ks_n = KP / 16;
       for (int prod = 0; prod < 3; ++prod) {
         const uint32_t aa = prod == 2 ? a_lo : a_hi, bb = prod == 1 ? b_lo : b_hi;
         for (int ks = 0; ks < ks_n; ++ks) {
@@ -417,6 +525,11 @@ __global__ void __launch_bounds__(kPjThreads, 1)
         }
       }
       tc::mma_commit(bar);
+    }
+    __syncwarp();
+    // ---- the next tile's pixels, while the MMAs run
+    if (t + step < ntiles) begin(t + step);
+    if (gt == 0) {
       const bool done = tc::mbar_wait_bounded(bar, iter & 1, kPjWaitNs);
       if (!done && err) atomicCAS(err, 0, RSC_ERR_TIMEOUT);
       s_ok[g] = done ? 1 : 0;
@@ -427,30 +540,40 @@ __global__ void __launch_bounds__(kPjThreads, 1)
       alive = false;
       break;
     }
-    // ---- read back and write the half spectrum, 32 columns at a time
+    // ---- read back; the tile's half spectra, one contiguous piece of the
+    // output, go out through the A area (free now) in one bulk copy
     const float unscale = ldexpf(1.0f, -(sa + sb));
-    float *out = coef + (p < P_total ? p : 0) * nout;
-    for (int piece = 0; piece * 32 < NP; ++piece) {
-      uint32_t v[32];
-      tc::tmem_ld32(dcol + lane_base + piece * 32, v);
+    float *so = reinterpret_cast<float *>(sA) + row * nout;
+    for (int piece = half; piece * 16 < NP; piece += 2) {
+      uint32_t d[16];
+      tc::tmem_ld16(dcol + lane_base + piece * 16, d);
       tc::tmem_wait_ld();
-      if (p < P_total) {
 #pragma unroll
-        for (int u = 0; u < 32; u += 4) {
-          const int o = piece * 32 + u;
-          if (o < nout)
-            *reinterpret_cast<float4 *>(out + o) =
-                make_float4(__uint_as_float(v[u]) * unscale, __uint_as_float(v[u + 1]) * unscale,
-                            __uint_as_float(v[u + 2]) * unscale,
-                            __uint_as_float(v[u + 3]) * unscale);
-        }
+      for (int u = 0; u < 16; u += 4) {
+        const int o = piece * 16 + u;
+        if (o < nout)
+          *reinterpret_cast<float4 *>(so + o) =
+              make_float4(__uint_as_float(d[u]) * unscale, __uint_as_float(d[u + 1]) * unscale,
+                          __uint_as_float(d[u + 2]) * unscale, __uint_as_float(d[u + 3]) * unscale);
       }
     }
     tc::fence_before_sync();
+    tc::fence_proxy_async_smem();
+    group_sync(g);
+    if (gt == 0) {
+      const int64_t p0 = t * kPjRows;
+      const uint32_t bytes = (uint32_t)(min((int64_t)kPjRows, P_total - p0) * nout * 4);
+      asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(
+                       coef + p0 * nout),
+                   "r"(tc::smem_u32(sA)), "r"(bytes)
+                   : "memory");
+      asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+    }
   }
+  if (gt == 0) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
   // a group whose wait gave up may still have MMAs in flight: wait (bounded)
   // before the accumulator columns are released
-  if (!alive && row == 0) tc::mbar_wait_bounded(bar, (iter & 1), kPjWaitNs);
+  if (!alive && gt == 0) tc::mbar_wait_bounded(bar, (iter & 1), kPjWaitNs);
   tc::fence_before_sync();
   __syncthreads();
   tc::fence_after_sync();
@@ -734,14 +857,18 @@ int launch_project(const rsc_basis *b, const ImageItem *items_dev, int n_items, 
   cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, b->device);
   if (b->Bt && (reinterpret_cast<uintptr_t>(coef) & 15) == 0) {
     const int total = pj_layout(b->NP).total;
-    cudaError_t e = cudaFuncSetAttribute(project_tc_kernel,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, total);
+    // one instantiation per 16 padded pixels (KP <= 128)
+    static constexpr decltype(&project_tc_kernel<1>) kernels[] = {
+        project_tc_kernel<1>, project_tc_kernel<2>, project_tc_kernel<3>, project_tc_kernel<4>,
+        project_tc_kernel<5>, project_tc_kernel<6>, project_tc_kernel<7>, project_tc_kernel<8>};
+    const auto kern = kernels[b->KP / 16 - 1];
+    cudaError_t e =
+        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, total);
     if (e != cudaSuccess) return rsc_cuda_fail(e);
     const int64_t tile_pairs = ((P_total + kPjRows - 1) / kPjRows + 1) / 2;
     const unsigned grid = (unsigned)std::min<int64_t>(tile_pairs, (int64_t)nsm);
-    project_tc_kernel<<<grid, kPjThreads, total, st>>>(items_dev, n_items, P_total, b->N,
-                                                        b->npix, b->offs, b->Bt, b->KP, b->NP,
-                                                        b->sb, b->nout, coef, b->err);
+    kern<<<grid, kPjThreads, total, st>>>(items_dev, n_items, P_total, b->N, b->npix, b->offs,
+                                          b->Bt, b->NP, b->sb, b->nout, coef, b->err);
     e = cudaGetLastError();
     return e == cudaSuccess ? RSC_OK : rsc_cuda_fail(e);
   }
