@@ -585,27 +585,55 @@ __global__ void __launch_bounds__(kPjThreads, 1)
 // split operator (hi and lo fp16, [2][256 outputs][KPw pixels], packed output
 // order, times 2^sbw) is too large for shared memory, so it streams from L2
 // one 64-pixel K-block at a time.  Per CTA and tile of 128 windows:
-//   * warps 0-3 (one thread per window) gather each K-block's 64 pixels,
-//     scaled by 2^sa and split into hi and lo, into 128-byte-swizzled K-major
-//     rows of a 2-stage A ring, then read the accumulator back and write the
-//     half spectrum;
-//   * warp 4 (one lane) loads the operator's K-block (hi and lo, 64 KB) into
+//   * warps 0-7 (two threads per window) find the window's scale in a first
+//     pass over its pixels (offsets from a table), then gather each K-block's
+//     64 pixels, scaled by 2^sa and split into hi and lo, into 128-byte-swizzled
+//     K-major rows of a 2-stage A ring;
+//   * warps 8-11 read the accumulator back and write the half spectra, 32
+//     columns at a time through shared memory so that stores run along rows;
+//   * warp 12 (one lane) loads the operator's K-block (hi and lo, 64 KB) into
 //     a 2-stage B ring with TMA;
-//   * warp 5 (one lane) issues hi*hi + hi*lo + lo*hi (3 x 4 MMAs, M = 128,
-//     N = 256) per K-block into one 256-column TMEM accumulator.
-// The gather warps' TMEM reads of tile t finish before they hand over the
-// first A block of tile t + 1 (tcgen05 fences around that mbarrier), so the
-// accumulator needs no second handshake.  Every wait is bounded.
-constexpr int kPwThreads = 192;
+//   * warp 13 (one lane) issues hi*hi + hi*lo + lo*hi (3 MMAs, M = 128, N =
+//     256, per 16 pixels that hold any) into one of two 256-column TMEM
+//     accumulators.
+// Floor: the MMAs (66 of 128 cycles a tile at 349 pixels, 61 us for 290,000
+// windows); bound by the gather's loads beside them (tensor pipe 29%).  290,000
+// windows of 21 x 21: 0.70 -> 0.24 ms against four gather warps that also wrote
+// the outputs, one float at a time from every row, with one accumulator.
+// Every wait is bounded.
+constexpr int kPwGather = 256;
+constexpr int kPwThreads = kPwGather + 6 * 32;
 constexpr int kPwBlkA = 128 * 128;     // one part (hi or lo) of an A K-block (bytes)
 constexpr int kPwStageA = 2 * kPwBlkA;
 constexpr int kPwBlkB = 256 * 128;     // one part of a B K-block: 256 outputs x 64 px
 constexpr int kPwStageB = 2 * kPwBlkB;
 constexpr int kPwStages = 2;
 constexpr int kPwNP = 256;             // MMA N: packed outputs, padded
-constexpr int kPwBarOff = kPwStages * (kPwStageA + kPwStageB);
+constexpr int kPwOutLd = 33;           // row pitch of a staged 32 x 32 piece (floats)
+constexpr int kPwSaRing = 4;           // tiles whose scales are kept
+constexpr int kPwOutOff = kPwStages * (kPwStageA + kPwStageB);
+constexpr int kPwOffOff = kPwOutOff + 4 * 32 * kPwOutLd * 4;
+constexpr int kPwMaxOff = kPwOffOff + 512 * 4;
+constexpr int kPwSaOff = kPwMaxOff + kPwGather * 4;
+constexpr int kPwBarOff = kPwSaOff + kPwSaRing * 128 * 4;
 constexpr int kPwSmem = kPwBarOff + 128 + 1024;
-enum : int { kPwAFull = 0, kPwAEmpty = 2, kPwBFull = 4, kPwBEmpty = 6, kPwAcc = 8, kPwBars = 9 };
+// barrier slots; two stages or accumulators each
+enum : int { kPwAFull = 0, kPwAEmpty = 2, kPwBFull = 4, kPwBEmpty = 6, kPwAccFull = 8, kPwAccEmpty = 10, kPwBars = 12 };
+static_assert(kPwBars * 8 + 8 <= 128 && kPwBarOff % 8 == 0, "barrier area");
+
+// Barrier of the gather warps; true for all of them when any has `p`.
+__device__ __forceinline__ bool gather_any(bool p) {
+  uint32_t r;
+  asm volatile(
+      "{\n\t.reg .pred a, b;\n\t"
+      "setp.ne.u32 a, %1, 0;\n\t"
+      "barrier.red.or.pred b, 1, %2, a;\n\t"
+      "selp.u32 %0, 1, 0, b;\n\t}"
+      : "=r"(r)
+      : "r"((uint32_t)p), "n"(kPwGather)
+      : "memory");
+  return r != 0;
+}
 
 __global__ void __launch_bounds__(kPwThreads, 1)
     project_tcw_kernel(const __grid_constant__ CUtensorMap tmW, const ImageItem *items,
@@ -616,24 +644,32 @@ __global__ void __launch_bounds__(kPwThreads, 1)
       (reinterpret_cast<uintptr_t>(pw_raw) + 1023) & ~uintptr_t(1023));
   unsigned char *sA = smem;
   unsigned char *sB = smem + kPwStages * kPwStageA;
+  int *s_off = reinterpret_cast<int *>(smem + kPwOffOff);
+  float *s_max = reinterpret_cast<float *>(smem + kPwMaxOff);
+  volatile int *s_sa = reinterpret_cast<volatile int *>(smem + kPwSaOff);
   uint64_t *bars = reinterpret_cast<uint64_t *>(smem + kPwBarOff);
   uint32_t *s_tmem = reinterpret_cast<uint32_t *>(bars + kPwBars);
   volatile int *s_abort = reinterpret_cast<volatile int *>(bars + kPwBars) + 1;
   const uint32_t bar0 = tc::smem_u32(bars);
   auto bar = [&](int i) { return bar0 + 8u * (uint32_t)i; };
+  auto arrive = [&](int i) {
+    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar(i)) : "memory");
+  };
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int nks = (npix + 15) / 16;  // 16-pixel steps that hold pixels
   if (tid == 0) {
-    for (int i = 0; i < kPwStages; ++i) {
-      tc::mbar_init(bar(kPwAFull + i), 4);  // one arrival per gather warp
+    for (int i = 0; i < 2; ++i) {
+      tc::mbar_init(bar(kPwAFull + i), kPwGather / 32);  // one arrival per gather warp
       tc::mbar_init(bar(kPwAEmpty + i), 1);
       tc::mbar_init(bar(kPwBFull + i), 1);
       tc::mbar_init(bar(kPwBEmpty + i), 1);
+      tc::mbar_init(bar(kPwAccFull + i), 1);
+      tc::mbar_init(bar(kPwAccEmpty + i), 4);  // one arrival per epilogue warp
     }
-    tc::mbar_init(bar(kPwAcc), 1);
     *s_abort = 0;
     tc::fence_mbar_init();
   }
-  if (warp == 0) tc::tmem_alloc(tc::smem_u32(s_tmem), kPwNP);
+  if (warp == 0) tc::tmem_alloc(tc::smem_u32(s_tmem), 2 * kPwNP);
   tc::fence_before_sync();
   __syncthreads();
   tc::fence_after_sync();
@@ -644,7 +680,7 @@ __global__ void __launch_bounds__(kPwThreads, 1)
     if (err) atomicCAS(err, 0, RSC_ERR_TIMEOUT);
   };
 
-  if (warp == 4) {
+  if (warp == 12) {
     // ------------------------------------------------------------ TMA (B)
     if (lane == 0) {
       uint32_t gj = 0;
@@ -667,13 +703,19 @@ __global__ void __launch_bounds__(kPwThreads, 1)
       for (uint32_t i = (gj > (uint32_t)kPwStages ? gj - kPwStages : 0); i < gj; ++i)
         tc::mbar_wait_bounded(bar(kPwBFull + i % kPwStages), (i / kPwStages) & 1, kPjWaitNs);
     }
-  } else if (warp == 5) {
+  } else if (warp == 13) {
     // ------------------------------------------------------------ MMA
     if (lane == 0) {
       const uint32_t idesc = tc::idesc_f16_f32(128, kPwNP);
-      uint32_t gj = 0, last = 0;
+      uint32_t gj = 0, it = 0, last = 0;
       bool any = false, ok = true;
-      for (int64_t t = blockIdx.x; ok && t < ntiles && !*s_abort; t += gridDim.x) {
+      for (int64_t t = blockIdx.x; ok && t < ntiles && !*s_abort; t += gridDim.x, ++it) {
+        const uint32_t b = it & 1, ub = it >> 1;
+        if (ub > 0 && !tc::mbar_wait_bounded(bar(kPwAccEmpty + b), (ub - 1) & 1, kPjWaitNs)) {
+          fail();
+          break;
+        }
+        const uint32_t d = tmem + b * kPwNP;
         for (int j = 0; j < nkb; ++j, ++gj) {
           const int s = (int)(gj % kPwStages);
           const uint32_t par = (gj / kPwStages) & 1;
@@ -686,128 +728,145 @@ __global__ void __launch_bounds__(kPwThreads, 1)
           tc::fence_after_sync();
           const uint32_t a_hi = tc::smem_u32(sA + s * kPwStageA), a_lo = a_hi + kPwBlkA;
           const uint32_t b_hi = tc::smem_u32(sB + s * kPwStageB), b_lo = b_hi + kPwBlkB;
+          const int steps = min(4, nks - 4 * j);
           for (int prod = 0; prod < 3; ++prod) {
             const uint32_t aa = prod == 2 ? a_lo : a_hi, bb = prod == 1 ? b_lo : b_hi;
-            for (int ks = 0; ks < 4; ++ks)
-              tc::mma_f16(tmem, tc::smem_desc_sw128(aa + ks * 32), tc::smem_desc_sw128(bb + ks * 32),
+            for (int ks = 0; ks < steps; ++ks)
+              tc::mma_f16(d, tc::smem_desc_sw128(aa + ks * 32), tc::smem_desc_sw128(bb + ks * 32),
                           idesc, (j | prod | ks) ? 1u : 0u);
           }
           tc::mma_commit(bar(kPwAEmpty + s));
           tc::mma_commit(bar(kPwBEmpty + s));
           last = gj;
           any = true;
-          if (j == nkb - 1) tc::mma_commit(bar(kPwAcc));
+          if (j == nkb - 1) tc::mma_commit(bar(kPwAccFull + b));
         }
       }
       // every MMA is followed by its stage's commit: the last one covers all
       if (any)
         tc::mbar_wait_bounded(bar(kPwAEmpty + last % kPwStages), (last / kPwStages) & 1, kPjWaitNs);
     }
-  } else if (warp < 4) {
-    // ------------------------------------------------ gather and epilogue
-    const int row = tid;
-    const uint32_t lane_base = (uint32_t)(warp * 32) << 16;
+  } else if (warp < 8) {
+    // ------------------------------------------------------------ gather
+    const int row = tid & 127, half = tid >> 7;
+    PixelOffsets px{s_off, offs, 0, npix, false};
+    int tab_w = -1;
     uint32_t gj = 0, it = 0;
     bool ok = true;
-    for (int64_t t = blockIdx.x; ok && t < ntiles; t += gridDim.x, ++it) {
-      const int64_t p = t * 128 + row;
-      const float *base = nullptr;
-      int w = 0;
-      float amax = 0.0f;
-      if (p < P_total) {
-        int lo = 0, hi = n_items - 1;  // last item with first <= p
-        while (lo < hi) {
-          const int mid = (lo + hi + 1) >> 1;
-          if (items[mid].first <= p) lo = mid; else hi = mid - 1;
+    for (int64_t t = blockIdx.x; t < ntiles; t += gridDim.x, ++it) {
+      const int64_t p0 = t * 128, last = min(p0 + 128, P_total) - 1;
+      const float *base = find_window(items, n_items, N, p0, last, p0 + row, px.w, px.one);
+      if (px.one && px.w != tab_w) {  // the same for all gather threads
+        gather_any(false);            // the previous table is read
+        for (int q = tid; q < 64 * nkb; q += kPwGather) {
+          const int2 o = __ldg(offs + (q < npix ? q : 0));
+          s_off[q] = o.x * px.w + o.y;
         }
-        const ImageItem itm = items[lo];
-        const int64_t local = p - itm.first;
-        const int nw = itm.w - N + 1;
-        const int r0 = (int)(local / nw), c0 = (int)(local - (int64_t)r0 * nw);
-        base = itm.img + (int64_t)r0 * itm.w + c0;
-        w = itm.w;
-        for (int q = 0; q < npix; ++q) {
-          const int2 o = __ldg(offs + q);
-          amax = fmaxf(amax, fabsf(__ldg(base + (int64_t)o.x * w + o.y)));
-        }
+        tab_w = px.w;
+        gather_any(false);
       }
-      int ea = 0;
-      (void)frexpf(amax, &ea);
-      const int sa = 14 - (ea < -100 ? -100 : (ea > 127 ? 127 : ea));  // max |x| 2^sa < 2^14
-      const float scale = ldexpf(1.0f, sa);
+      float amax = 0.0f;
+#pragma unroll 4
+      for (int q = 8 * half; q < npix; q += 16) {
+        float v[8];
+        px.load<8>(base, q, v);
+#pragma unroll
+        for (int u = 0; u < 8; ++u) amax = fmaxf(amax, fabsf(v[u]));
+      }
+      s_max[tid] = amax;
+      // a wait that gave up in the last tile ends all gather warps here
+      if (gather_any(!ok)) break;
+      const int sa = pixel_scale(fmaxf(s_max[row], s_max[row + 128]));
+      const float scale = __int_as_float((sa + 127) << 23);  // 2^sa, |sa| < 126
+      // (a slot is written again four tiles on, when the epilogue that read
+      // it is done: the MMAs of the tile before need its accumulator)
+      if (half == 0) s_sa[(it % kPwSaRing) * 128 + row] = sa;
       for (int j = 0; j < nkb; ++j, ++gj) {
         const int s = (int)(gj % kPwStages);
-        const bool done = !*s_abort && (gj < (uint32_t)kPwStages ||
-                                        tc::mbar_wait_bounded(bar(kPwAEmpty + s),
-                                                              ((gj / kPwStages) - 1) & 1, kPjWaitNs));
+        // the block's pixels are on their way while the stage is waited for
+        float v[4][8];
+        const int q0 = 64 * j + 32 * half;
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+          if (q0 + 8 * i < npix) px.load<8>(base, q0 + 8 * i, v[i]);
+        const bool done = ok && !*s_abort &&
+                          (gj < (uint32_t)kPwStages ||
+                           tc::mbar_wait_bounded(bar(kPwAEmpty + s), ((gj / kPwStages) - 1) & 1,
+                                                 kPjWaitNs));
         if (!__all_sync(0xffffffffu, done)) {
           if (lane == 0) fail();
           ok = false;
           break;
         }
         unsigned char *dst = sA + s * kPwStageA;
-        for (int c = 0; c < 8; ++c) {
-          uint32_t hv[4], lv[4];
 #pragma unroll
-          for (int u = 0; u < 4; ++u) {
-            float x2[2];
-#pragma unroll
-            for (int h = 0; h < 2; ++h) {
-              const int q = j * 64 + c * 8 + 2 * u + h;
-              float x = 0.0f;
-              if (base && q < npix) {
-                const int2 o = __ldg(offs + q);
-                x = __ldg(base + (int64_t)o.x * w + o.y) * scale;
-              }
-              x2[h] = x;
-            }
-            const __half2 hh = __floats2half2_rn(x2[0], x2[1]);
-            const float2 hf = __half22float2(hh);
-            const __half2 ll = __floats2half2_rn(x2[0] - hf.x, x2[1] - hf.y);
-            hv[u] = *reinterpret_cast<const uint32_t *>(&hh);
-            lv[u] = *reinterpret_cast<const uint32_t *>(&ll);
+        for (int i = 0; i < 4; ++i) {
+          const int c = 4 * half + i, q = q0 + 8 * i;
+          if (q < 16 * nks) {
+            uint4 hi = make_uint4(0, 0, 0, 0), lo = hi;
+            if (q < npix) split8<true>(v[i], q, npix, scale, hi, lo);
+            const int off = row * 128 + ((c ^ (row & 7)) << 4);
+            *reinterpret_cast<uint4 *>(dst + off) = hi;
+            *reinterpret_cast<uint4 *>(dst + kPwBlkA + off) = lo;
           }
-          const int off = row * 128 + ((c ^ (row & 7)) << 4);
-          *reinterpret_cast<uint4 *>(dst + off) = make_uint4(hv[0], hv[1], hv[2], hv[3]);
-          *reinterpret_cast<uint4 *>(dst + kPwBlkA + off) = make_uint4(lv[0], lv[1], lv[2], lv[3]);
         }
         tc::fence_proxy_async_smem();
         tc::fence_before_sync();
         __syncwarp();
-        if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar(kPwAFull + s)) : "memory");
+        if (lane == 0) arrive(kPwAFull + s);
       }
-      if (!ok) break;
-      // ---- read the accumulator back: packed output q -> half spectrum
-      // index 2q (q < J: Re of k = 0, whose Im is 0) or J + q
-      const bool done = !*s_abort && tc::mbar_wait_bounded(bar(kPwAcc), it & 1, kPjWaitNs);
+      // the pair's maxima are read before the next tile's are written
+      if (gather_any(!ok)) break;
+    }
+  } else {
+    // ---------------------------------------------------------- epilogue
+    const int quarter = warp & 3;
+    const uint32_t lane_base = (uint32_t)(quarter * 32) << 16;
+    float *s_out = reinterpret_cast<float *>(smem + kPwOutOff) + quarter * 32 * kPwOutLd;
+    uint32_t it = 0;
+    for (int64_t t = blockIdx.x; t < ntiles; t += gridDim.x, ++it) {
+      const uint32_t b = it & 1;
+      const bool done =
+          !*s_abort && tc::mbar_wait_bounded(bar(kPwAccFull + b), (it >> 1) & 1, kPjWaitNs);
       if (!__all_sync(0xffffffffu, done)) {
         if (lane == 0) fail();
         break;
       }
       tc::fence_after_sync();
-      const float unscale = ldexpf(1.0f, -(sa + sb));
-      float *out = coef + (p < P_total ? p : 0) * nout;
-      for (int piece = 0; piece * 32 < n; ++piece) {
+      const float unscale =
+          ldexpf(1.0f, -(s_sa[(it % kPwSaRing) * 128 + quarter * 32 + lane] + sb));
+      const int64_t w0 = t * 128 + quarter * 32;
+      const int rows = (int)max((int64_t)0, min((int64_t)32, P_total - w0));
+      float *out = coef + w0 * nout;
+      for (int c0 = 0; c0 < n; c0 += 32) {
         uint32_t v[32];
-        tc::tmem_ld32(tmem + lane_base + piece * 32, v);
+        tc::tmem_ld32(tmem + lane_base + b * kPwNP + c0, v);
         tc::tmem_wait_ld();
-        if (p < P_total) {
 #pragma unroll
-          for (int u = 0; u < 32; ++u) {
-            const int q = piece * 32 + u;
-            if (q < n) out[q < J ? 2 * q : J + q] = __uint_as_float(v[u]) * unscale;
-          }
+        for (int u = 0; u < 32; ++u) s_out[lane * kPwOutLd + u] = __uint_as_float(v[u]) * unscale;
+        __syncwarp();
+        // packed output q -> half spectrum index 2q (q < J: Re of k = 0,
+        // whose Im is 0) or J + q
+        const int q = c0 + lane;
+        if (q < n) {
+          float *o = out + (q < J ? 2 * q : J + q);
+          const float *si = s_out + lane;
+#pragma unroll 8
+          for (int r = 0; r < rows; ++r) o[(int64_t)r * nout] = si[r * kPwOutLd];
+          if (q < J)
+            for (int r = 0; r < rows; ++r) o[(int64_t)r * nout + 1] = 0.0f;
         }
+        __syncwarp();
       }
-      if (p < P_total)
-        for (int jj = 0; jj < J; ++jj) out[2 * jj + 1] = 0.0f;
       tc::fence_before_sync();
+      __syncwarp();
+      if (lane == 0) arrive(kPwAccEmpty + b);
     }
   }
   tc::fence_before_sync();
   __syncthreads();
   tc::fence_after_sync();
-  if (warp == 0) tc::tmem_dealloc(tmem, kPwNP);
+  if (warp == 0) tc::tmem_dealloc(tmem, 2 * kPwNP);
 }
 
 // Multi-dictionary labelling (the paper's classifier, Sec. III-B): after
