@@ -155,6 +155,17 @@ __device__ __forceinline__ uint64_t smem_desc_sw128(uint32_t saddr) {
   return d;
 }
 
+// A descriptor `bytes` further on (a multiple of 16): the start address is the
+// low field, so one 32-bit addition; building a descriptor anew for every MMA
+// costs the issuing thread more than the MMA takes.
+__device__ __forceinline__ uint64_t desc_at(uint64_t desc, uint32_t bytes) {
+  uint32_t lo, hi;
+  asm("mov.b64 {%0, %1}, %2;" : "=r"(lo), "=r"(hi) : "l"(desc));
+  uint64_t r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "r"(lo + (bytes >> 4)), "r"(hi));
+  return r;
+}
+
 // Instruction descriptor of kind::f16: fp16 A and B (format code 0 in bits
 // 7-9 and 10-12, both operands the same type), K-major, f32 D (bits 4-5 = 1),
 // N >> 3 in bits 17-22, M >> 4 in bits 24-28.
