@@ -175,6 +175,7 @@ __global__ void __launch_bounds__(kSThreads, 1)
   } else if (warp == kSEpi + 1) {
     // ---------------------------------------------------------------- MMA
     if (lane == 0) {
+      const uint64_t bs0 = tc::smem_desc_sw128(tc::smem_u32(sB));
       uint32_t g = 0, gs = 0, it = 0, last = 0;
       bool any = false, ok = true;
       for (int64_t tile = blockIdx.x; ok && tile < ntiles && !*s_abort; tile += gridDim.x, ++it) {
@@ -185,7 +186,7 @@ __global__ void __launch_bounds__(kSThreads, 1)
           break;
         }
         tc::fence_after_sync();
-        const uint32_t a0 = tc::smem_u32(sA + ab * Sh::kATile);
+        const uint64_t a0 = tc::smem_desc_sw128(tc::smem_u32(sA + ab * Sh::kATile));
         for (int c = 0; c < nch; ++c, ++g) {
           const uint32_t b = g & 1, ub = g >> 1;
           if (ub > 0 && !tc::mbar_wait_bounded(bar(kBarAccEmpty + b), (ub - 1) & 1, a.wait_ns)) {
@@ -194,6 +195,7 @@ __global__ void __launch_bounds__(kSThreads, 1)
           }
           tc::fence_after_sync();
           const uint32_t d = tmem + b * kSBufC;
+#pragma unroll
           for (int j = 0; j < NKB; ++j, ++gs) {
             const int s = (int)(gs % kStages);
             if (!tc::mbar_wait_bounded(bar(kBarBFull + s), (gs / kStages) & 1, a.wait_ns)) {
@@ -201,21 +203,16 @@ __global__ void __launch_bounds__(kSThreads, 1)
               break;
             }
             tc::fence_after_sync();
-            const uint32_t b0 = tc::smem_u32(sB + s * Sh::kBStage);
-            const uint32_t aj = a0 + j * kABlk;
-            if (PAIRED) {
-              // block 0: even harmonics -> columns 0..N-1 of the buffer;
-              // block 1: odd harmonics -> columns N..2N-1
-              const int nk = j == 0 ? a.ke : a.ko;
-              for (int ks = 0; ks < nk; ++ks)
-                tc::mma_f16(d + (uint32_t)(j * N), tc::smem_desc_sw128(aj + ks * 32),
-                            tc::smem_desc_sw128(b0 + ks * 32), kIdesc, ks > 0 ? 1u : 0u);
-            } else {
-              const int nk = min(4, a.ksteps - 4 * j);
-              for (int ks = 0; ks < nk; ++ks)
-                tc::mma_f16(d, tc::smem_desc_sw128(aj + ks * 32), tc::smem_desc_sw128(b0 + ks * 32),
-                            kIdesc, (j > 0 || ks > 0) ? 1u : 0u);
-            }
+            const uint64_t b0 = tc::desc_at(bs0, (uint32_t)(s * Sh::kBStage));
+            // paired: block 0 holds the even harmonics -> columns 0..N-1 of
+            // the buffer, block 1 the odd ones -> columns N..2N-1
+            const int nk = PAIRED ? (j == 0 ? a.ke : a.ko) : a.ksteps - 4 * j;
+#pragma unroll
+            for (int ks = 0; ks < 4; ++ks)
+              if (ks < nk)
+                tc::mma_f16(PAIRED ? d + (uint32_t)(j * N) : d, tc::desc_at(a0, j * kABlk + ks * 32),
+                            tc::desc_at(b0, ks * 32), kIdesc,
+                            (PAIRED ? ks > 0 : j > 0 || ks > 0) ? 1u : 0u);
             tc::mma_commit(bar(kBarBEmpty + s));
             last = gs;
             any = true;
