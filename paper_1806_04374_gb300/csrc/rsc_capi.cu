@@ -13,6 +13,7 @@
 #include <string>
 #include <vector>
 
+#include "df.cuh"
 #include "rsc_internal.h"
 #include "rsc_trace.h"
 
@@ -143,10 +144,7 @@ void free_dict(rsc_dict *d) {
   cudaFree(d->fallbacks);
   cudaFree(d->steered_f16);
   cudaFree(d->paired_f16);
-  cudaFree(d->xgram);
-  cudaFree(d->anorm);
-  cudaFree(d->rows);
-  cudaFree(d->gram);
+  cudaFree(d->xgram);  // and the tables behind it
   delete d;
 }
 
@@ -186,11 +184,14 @@ int encode_rows_map(CUtensorMap *map, void *base, size_t rows, int box_rows, int
 }
 
 // Packed steered rows (rsc_slot_code layout): entry q of row r*M + m,
-// r < nR, is slot q of kDictScale S_r d_m in fp16, computed in FP64 from the
-// atoms; the angle k r 2 pi / R is reduced exactly (k r mod R).
-__global__ void steered_rows_kernel(const float *__restrict__ d, int M, int J, int kmax, int R,
-                                    int nR, int L, int paired, uint16_t *out) {
-  const int HJ = (kmax + 1) * J;
+// r < nR, is slot q of kDictScale S_r d_m in fp16, rounded once from the atoms
+// and the double-float steering factors.  (FP64, with a sine and a cosine an
+// entry, held this up: 872 us for M = 256, R = 128, L = 256 before.)
+__global__ void steered_rows_kernel(const float *__restrict__ d, const float *__restrict__ tw,
+                                    int M, int J, int kmax, int R, int nR, int L, int paired,
+                                    uint16_t *out) {
+  const int H = kmax + 1, HJ = H * J;
+  const df sqrt2 = {1.41421354f, 2.42032346e-08f};
   const int64_t total = (int64_t)nR * M * L;
   for (int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; idx < total;
        idx += (int64_t)gridDim.x * blockDim.x) {
@@ -201,12 +202,15 @@ __global__ void steered_rows_kernel(const float *__restrict__ d, int M, int J, i
     uint16_t bits = 0;
     if (code >= 0) {
       const int e = code >> 8, k = (code >> 1) & 127, c = code & 1;
-      const double th = 2.0 * M_PI * (double)(int)(((int64_t)k * r) % R) / (double)R;
-      const double co = cos(th), si = sin(th);
-      const double dre = d[((size_t)m * HJ + e) * 2];
-      const double dim = k ? (double)d[((size_t)m * HJ + e) * 2 + 1] : 0.0;
-      const double re = co * dre + si * dim, im = co * dim - si * dre;  // e^{-ik theta} d
-      const double v = (k == 0 ? re : M_SQRT2 * (c ? im : re)) * (double)kDictScale;
+      const df co = {tw[(0 * H + k) * R + r], tw[(1 * H + k) * R + r]};
+      const df si = {tw[(2 * H + k) * R + r], tw[(3 * H + k) * R + r]};
+      const float dre = d[((size_t)m * HJ + e) * 2];
+      const float dim = k ? d[((size_t)m * HJ + e) * 2 + 1] : 0.0f;
+      // e^{-ik theta} d
+      df y = c ? df_sub(df_mul_f(co, dim), df_mul_f(si, dre))
+               : df_add(df_mul_f(co, dre), df_mul_f(si, dim));
+      if (k) y = df_mul(y, sqrt2);
+      const double v = df_to_d(y) * (double)kDictScale;
       const __half hv = __double2half(v);
       bits = *reinterpret_cast<const uint16_t *>(&hv);
     }
@@ -270,8 +274,8 @@ __global__ void refine_rows_kernel(const float *__restrict__ d, const float *__r
 }
 
 // Gram entries of steered atoms, <S_r d_a, d_b> = sum_k w_k Re(e^{ik theta_r}
-// H_k(a, b)) in FP64 from the cross-Gram table, stored as double-float at
-// [(a M + b) R + r].
+// H_k(a, b)) in double-float from the cross-Gram table, at [(a M + b) R + r].
+// (In FP64, at 64 cycles an instruction, M = 256, R = 128, H = 13 took 3.1 ms.)
 __global__ void gram_kernel(const float4 *__restrict__ X, const float *__restrict__ tw, int M,
                             int H, int R, float2 *__restrict__ G) {
   const int64_t total = (int64_t)M * M * R;
@@ -279,16 +283,15 @@ __global__ void gram_kernel(const float4 *__restrict__ X, const float *__restric
        idx += (int64_t)gridDim.x * blockDim.x) {
     const int r = (int)(idx % R);
     const float4 *h = X + (idx / R) * H;
-    double g = 0.0;
+    df g = df_make(0.0f);
     for (int k = 0; k < H; ++k) {
       const float4 v = __ldg(h + k);
-      const double co = (double)tw[(0 * H + k) * R + r] + (double)tw[(1 * H + k) * R + r];
-      const double si = (double)tw[(2 * H + k) * R + r] + (double)tw[(3 * H + k) * R + r];
-      const double t = co * ((double)v.x + (double)v.y) - si * ((double)v.z + (double)v.w);
-      g += k ? 2.0 * t : t;
+      const df co = {tw[(0 * H + k) * R + r], tw[(1 * H + k) * R + r]};
+      const df si = {tw[(2 * H + k) * R + r], tw[(3 * H + k) * R + r]};
+      const df t = df_sub(df_mul(co, df{v.x, v.y}), df_mul(si, df{v.z, v.w}));
+      g = df_add(g, k ? df{2.0f * t.hi, 2.0f * t.lo} : t);
     }
-    const float hi = (float)g;
-    G[idx] = make_float2(hi, (float)(g - (double)hi));
+    G[idx] = make_float2(g.hi, g.lo);
   }
 }
 
@@ -333,26 +336,34 @@ int build_tc_tables(rsc_dict *d, cudaStream_t st) {
   }
   cudaError_t e = cudaMalloc(&d->steered_f16, rows * L * 2);
   if (e == cudaSuccess && paired) e = cudaMalloc(&d->paired_f16, rows / 2 * kTcKst * 2);
-  if (e == cudaSuccess) e = cudaMalloc(&d->xgram, (size_t)M * M * H * sizeof(float4));
-  if (e == cudaSuccess) e = cudaMalloc(&d->anorm, (size_t)M * sizeof(float2));
   d->Rr = R % 2 == 0 ? R / 2 : R;
   const int64_t nrow = (int64_t)d->Rr * M * L, ng = (int64_t)M * M * R;
-  if (e == cudaSuccess) e = cudaMalloc(&d->rows, (size_t)nrow * 2 * sizeof(float));
-  if (e == cudaSuccess && ng * sizeof(float2) <= kGramMax)
-    e = cudaMalloc(&d->gram, (size_t)ng * sizeof(float2));
+  // the refine's tables share one allocation, at d->xgram
+  auto al = [](size_t v) { return (v + 255) & ~(size_t)255; };
+  const size_t bx = al((size_t)M * M * H * sizeof(float4)), ba = al((size_t)M * sizeof(float2)),
+               br = al((size_t)nrow * 2 * sizeof(float)), bg = (size_t)ng * sizeof(float2);
+  const bool gram = bg <= kGramMax;
+  unsigned char *tables = nullptr;
+  if (e == cudaSuccess) e = cudaMalloc(&tables, bx + ba + br + (gram ? bg : 0));
+  if (e == cudaSuccess) {
+    d->xgram = reinterpret_cast<float4 *>(tables);
+    d->anorm = reinterpret_cast<float2 *>(tables + bx);
+    d->rows = reinterpret_cast<float *>(tables + bx + ba);
+    d->gram = gram ? reinterpret_cast<float2 *>(tables + bx + ba + br) : nullptr;
+  }
   if (e == cudaErrorMemoryAllocation) {
     cudaGetLastError();
     return RSC_ERR_OOM;
   }
   if (e != cudaSuccess) return rsc_cuda_fail(e);
-  // the tables are built on the device from the uploaded atoms (FP64 arithmetic)
+  // the tables are built on the device from the uploaded atoms (double-float or FP64)
   const int T = 256;
   const int64_t nb = (int64_t)rows * L, np = paired ? (int64_t)rows / 2 * kTcKst : 0;
   steered_rows_kernel<<<(unsigned)((nb + T - 1) / T), T, 0, st>>>(
-      d->d, M, J, d->kmax, R, R, L, 0, static_cast<uint16_t *>(d->steered_f16));
+      d->d, d->tw, M, J, d->kmax, R, R, L, 0, static_cast<uint16_t *>(d->steered_f16));
   if (paired)
     steered_rows_kernel<<<(unsigned)((np + T - 1) / T), T, 0, st>>>(
-        d->d, M, J, d->kmax, R, R / 2, kTcKst, 1, static_cast<uint16_t *>(d->paired_f16));
+        d->d, d->tw, M, J, d->kmax, R, R / 2, kTcKst, 1, static_cast<uint16_t *>(d->paired_f16));
   const int64_t nx = (int64_t)M * M * H;
   xgram_kernel<<<(unsigned)((nx + T - 1) / T), T, 0, st>>>(d->d, M, J, H, d->xgram);
   anorm_kernel<<<(M + T - 1) / T, T, 0, st>>>(d->d, M, J, H, d->anorm);
