@@ -6,21 +6,30 @@
 //   (a) per-harmonic contraction G_k(m) = sum_j conj(d_m[j,k]) r[j,k], one
 //       lane per atom, FP32 FMA, the residual broadcast from shared memory;
 //   (b) angle transform score(m, r) = G_0 + 2 Re sum_k e^{ik 2 pi r / R} G_k,
-//       one lane per angle with its cos/sin factors held in registers; with
-//       RSC_FP32_PRUNE only for the atoms whose exact bound |G_0| +
+//       one lane per angle, or per pair of angles half a turn apart, with its
+//       cos/sin factors held in registers; with RSC_FP32_PRUNE only for the atoms whose exact bound |G_0| +
 //       2 sum_k |G_k| >= max_r |score(m, r)| can still reach the window of
 //       the running best;
-//   (c) per-lane top-4 of |score| plus the largest discarded value, merged
-//       over the warp into every candidate within 2E of the best, where E
-//       bounds the FP32 error of a score; the candidates are re-scored in
-//       double-float arithmetic against the double-float residual (if a lane
-//       discarded a value inside the window, all M*R candidates are
-//       re-scored exactly instead);
+//   (c) per lane and angle the largest |score| and its runner-up, merged over
+//       the warp into every candidate within 2E of the best, where E bounds
+//       the FP32 error of a score; if a runner-up lies inside that window, the
+//       step's scores are computed again with a top-4 a lane and the largest
+//       discarded value.  The candidates are re-scored in double-float
+//       arithmetic against the double-float residual (if a lane discarded a
+//       value inside the window, all M*R candidates are re-scored exactly
+//       instead);
 //   (e) new row of the Cholesky factor of the Gram matrix of the selected
 //       steered atoms (entries and right-hand side in double-float, factor and
-//       solve in FP64 on lane 0);
+//       solve in FP64, a lane an entry);
 //   (d) residual x - sum_i a_i S_{r_i} d_{m_i} in double-float, its high part
 //       feeding the next scoring pass.
+//
+// Bound by instruction issue (80% of the slots, 6.2 thousand warp instructions
+// a patch and step at M = 64, R = 64, K = 5; the code's traffic is the input
+// once).  With a branching top-4 insert for every value, no pairs and the
+// factor on lane 0 it took 10.5 thousand at 59%: 100,003 patches 7.42 ms then,
+// 3.14 ms now.  The exact part's loops are kept rolled: unrolled, their code
+// overran the instruction cache (4.24 against 3.58 ms).
 #include <math.h>
 
 #include "df.cuh"
@@ -39,11 +48,11 @@ struct GStride {
 struct Layout {
   // block-level
   int tw_off, tw_stride;  // twiddles [4][H][tw_stride]
-  int dT_off;             // transposed atoms [2][HJ][M] or -1 (read from global)
+  int dT_off;             // transposed atoms [HJ][M] (re, im) or -1 (read from global)
   // per-warp
   int warp_off, warp_bytes;
   int x_off, rhi_off, rlo_off, g_off, ub_off, cand_off, L_off, inv_off, z_off, a_off, adf_off,
-      sel_off, gram_off;
+      sel_off;
   int acache_off;  // [K][HJ] float4: steered selected atoms (re hi, re lo, im hi, im lo)
   int total;
 };
@@ -75,7 +84,6 @@ __host__ __device__ inline Layout make_layout(int M, int J, int H, int R, int K,
   L.a_off = w;    w = align16(w + K * 8);
   L.adf_off = w;  w = align16(w + 2 * K * 4);
   L.sel_off = w;  w = align16(w + K * 4);
-  L.gram_off = w; w = align16(w + (2 * K + 2) * 8);
   L.acache_off = w; w = align16(w + K * HJ * 16);
   L.warp_bytes = w;
   L.total = off + warps * w;
@@ -152,8 +160,19 @@ __device__ __forceinline__ float4 cdf_pack(const Cdf &a) {
 
 __device__ __forceinline__ Cdf cdf_unpack(float4 v) { return {{v.x, v.y}, {v.z, v.w}}; }
 
+// PAIR (even R): a lane takes the angles r and r + R/2 together.  Half a turn
+// changes the sign of the odd harmonics only, so the even and odd parts of
+// score(m, r) give both values; RPL counts the lane's angles below R/2.
+// Warps of a block: where the angle factors leave room (96 registers), 20 that
+// share one copy of the tables, the most that shared memory takes at M = 64,
+// n = 102, K = 5 (3.13 ms there; 16 warps 3.33), else 8, twice an SM.
 template <int KM, int RPL, bool PRUNE>
-__global__ void __launch_bounds__(256)
+struct BlockWarps {
+  static constexpr int v = !PRUNE && KM == 8 && RPL == 1 ? 20 : 8;
+};
+
+template <int KM, int RPL, bool PAIR, bool PRUNE>
+__global__ void __launch_bounds__((32 * BlockWarps<KM, RPL, PRUNE>::v))
     romp_f32_kernel(RompArgs a, int dT_in_smem) {
   extern __shared__ __align__(16) unsigned char smem[];
   constexpr int GS = GStride<KM>::v;
@@ -173,10 +192,10 @@ __global__ void __launch_bounds__(256)
     int plane_k = i / R, r = i - plane_k * R;
     s_tw[plane_k * Lo.tw_stride + r] = a.tw[i];
   }
-  const float *dT = a.dT;
+  const float2 *dT = reinterpret_cast<const float2 *>(a.dT);
   if (dT_in_smem) {
-    float *s_dT = reinterpret_cast<float *>(smem + Lo.dT_off);
-    for (int i = threadIdx.x; i < 2 * HJ * M; i += blockDim.x) s_dT[i] = a.dT[i];
+    float2 *s_dT = reinterpret_cast<float2 *>(smem + Lo.dT_off);
+    for (int i = threadIdx.x; i < HJ * M; i += blockDim.x) s_dT[i] = dT[i];
     dT = s_dT;
   }
   __syncthreads();
@@ -195,17 +214,24 @@ __global__ void __launch_bounds__(256)
   double *s_a = reinterpret_cast<double *>(wbase + Lo.a_off);
   float *s_adf = reinterpret_cast<float *>(wbase + Lo.adf_off);
   int *s_sel = reinterpret_cast<int *>(wbase + Lo.sel_off);
-  double *s_gram = reinterpret_cast<double *>(wbase + Lo.gram_off);
   float4 *s_A = reinterpret_cast<float4 *>(wbase + Lo.acache_off);
 
   // FP32 angle factors of this lane's angles r = lane + 32 i, harmonics 1..KM
+  const int Rh = PAIR ? R / 2 : R;
+  constexpr int NV = PAIR ? 2 * RPL : RPL;  // angles of a lane
+  // angle of value v of the lane: r_of(v), if valid(v)
+  auto r_of = [&](int v) { return lane + 32 * (PAIR ? v >> 1 : v) + (PAIR && (v & 1) ? Rh : 0); };
+  auto valid = [&](int v) { return lane + 32 * (PAIR ? v >> 1 : v) < Rh; };
+  // e / J for e < kMaxEntries: 2^22 > e (J - 1), and no overflow
+  const uint32_t inv_J = ((1u << 22) + (uint32_t)J - 1u) / (uint32_t)J;
+  auto k_of = [&](int e) { return (int)(((uint32_t)e * inv_J) >> 22); };
   float tc[RPL][KM], ts[RPL][KM];
 #pragma unroll
   for (int i = 0; i < RPL; ++i) {
     int r = lane + 32 * i;
 #pragma unroll
     for (int k = 0; k < KM; ++k) {
-      bool ok = (r < R) && (k + 1 <= kmax);
+      bool ok = (r < Rh) && (k + 1 <= kmax);
       tc[i][k] = ok ? tw.cosv(k + 1, r).hi : 0.0f;
       ts[i][k] = ok ? tw.sinv(k + 1, r).hi : 0.0f;
     }
@@ -261,128 +287,186 @@ __global__ void __launch_bounds__(256)
         best_c = a.resume_sI[(int64_t)step * a.resume_P + p] * R +
                  a.resume_sI[(int64_t)(a.resume_cap + step) * a.resume_P + p];
       } else {
-        // ---- (a)+(b)+(c): FP32 scores, per-lane top-4
+        // ---- (a)+(b)+(c): FP32 scores.  First the largest value of each of
+        // the lane's angles, its atom and the runner-up, without branches; if
+        // a runner-up lies within the window (rare), again with a top-4 a lane.
+        float bv[NV], sv[NV];
+        int bm[NV];
+#pragma unroll
+        for (int v = 0; v < NV; ++v) {
+          bv[v] = sv[v] = -INFINITY;
+          bm[v] = -1;
+        }
         float tv[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
         int ti[4] = {-1, -1, -1, -1};
-        float disc = -INFINITY;
-        const float win2 = 2.0f * err_per_norm * rnorm;
-        for (int mc = 0; mc < M; mc += kChunk) {
-          const int mend = min(kChunk, M - mc);
-          // (a) one lane per atom: G_k = sum_j conj(d[j,k]) r[j,k]
-          for (int ml = lane; ml < mend; ml += 32) {
-            const int m = mc + ml;
-            float gv[GS];
-#pragma unroll
-            for (int q = 0; q < GS; ++q) gv[q] = 0.0f;
-            const float *pre = dT + m;
-            const float *pim = dT + (size_t)HJ * M + m;
-            const float2 *r2 = reinterpret_cast<const float2 *>(s_rhi);
-            int e = 0;
-#pragma unroll
-            for (int k = 0; k <= KM; ++k) {
-              if (k < H) {
-                float gre0 = 0.f, gre1 = 0.f, gim0 = 0.f, gim1 = 0.f;
-                for (int j = 0; j < J; ++j, ++e) {
-                  const float dre = pre[(size_t)e * M], dim = pim[(size_t)e * M];
-                  const float2 rv = r2[e];
-                  gre0 = fmaf(dre, rv.x, gre0);
-                  gre1 = fmaf(dim, rv.y, gre1);
-                  gim0 = fmaf(dre, rv.y, gim0);
-                  gim1 = fmaf(-dim, rv.x, gim1);
-                }
-                if (k == 0) {
-                  gv[0] = gre0 + gre1;
-                } else {
-                  gv[2 * k - 1] = 2.0f * (gre0 + gre1);
-                  gv[2 * k] = -2.0f * (gim0 + gim1);
-                }
-              }
-            }
-            float4 *g4 = reinterpret_cast<float4 *>(s_g + ml * GS);
-#pragma unroll
-            for (int q = 0; q < GS / 4; ++q)
-              g4[q] = make_float4(gv[4 * q], gv[4 * q + 1], gv[4 * q + 2], gv[4 * q + 3]);
-            if constexpr (PRUNE) {
-              // |score(m, r)| <= |G_0| + 2 sum_k |G_k| for every angle
-              // (triangle inequality; gv holds G_0 and 2 Re / -2 Im of G_k),
-              // times a slack covering the FP32 rounding of this sum and of
-              // the transform below, so every FP32 score of the atom is <= ub
-              float ub = fabsf(gv[0]);
-#pragma unroll
-              for (int k = 1; k <= KM; ++k)
-                if (k <= kmax) ub += sqrtf(fmaf(gv[2 * k - 1], gv[2 * k - 1], gv[2 * k] * gv[2 * k]));
-              s_ub[ml] = ub * (1.0f + 16.0f * (KM + 2) * 5.9604644775390625e-8f);
-            }
-          }
-          __syncwarp();
-          // (b) one lane per angle, (c) per-lane top-4
-          auto transform = [&](int ml) {
-            const float4 *g4 = reinterpret_cast<const float4 *>(s_g + ml * GS);
-            float gv[GS];
-#pragma unroll
-            for (int q = 0; q < GS / 4; ++q) {
-              float4 v = g4[q];
-              gv[4 * q] = v.x;
-              gv[4 * q + 1] = v.y;
-              gv[4 * q + 2] = v.z;
-              gv[4 * q + 3] = v.w;
-            }
-#pragma unroll
-            for (int i = 0; i < RPL; ++i) {
-              float sa = gv[0], sb = 0.0f;
-#pragma unroll
-              for (int k = 0; k < KM; ++k) {
-                sa = fmaf(gv[2 * k + 1], tc[i][k], sa);
-                sb = fmaf(gv[2 * k + 2], ts[i][k], sb);
-              }
-              const int r = lane + 32 * i;
-              const float v = fabsf(sa + sb);
-              // a value more than 2E below this lane's running best is below
-              // the final window and need not be kept (the best only grows)
-              if (r < R && !(v < tv[0] - win2)) top4_insert(tv, ti, disc, v, (mc + ml) * R + r);
-            }
-          };
-          if constexpr (!PRUNE) {
-            for (int ml = 0; ml < mend; ++ml) transform(ml);
-          } else {
-            // In index order, an atom whose bound is below the warp's running
-            // best minus the window 2E (refreshed every 8 atoms; a stale best
-            // is lower, so only more atoms are transformed) is skipped: every
-            // FP32 score of it is below best - 2E <= the final threshold
-            // s1 - 2E (the best only grows), so none of them could be a
-            // candidate or raise a lane's discarded value to the threshold;
-            // the best atom is never skipped (its bound is >= its score).
-            // Measured at M = 64, R = 64, K = 5 (400,000 patches): with the
-            // chunk's largest-bound atom first the bound rules out 52% of the
-            // transforms, yet that loop takes 1.55x the plain loop's time and
-            // this one 1.3x; the same loop transforming every atom takes
-            // 1.06x.  The plain loop's unbroken run of short FMA chains
-            // pipelines better than any loop with a data-dependent skip.
-            float wbest = -INFINITY;
-            for (int ml = 0; ml < mend; ++ml) {
-              if ((ml & 7) == 0) wbest = warp_max(tv[0]);
-              if (s_ub[ml] < wbest - win2) continue;
-              transform(ml);
-            }
-          }
-          __syncwarp();
-        }
-        const float s1 = warp_max(tv[0]);
+        float disc = -INFINITY, s1 = 0.0f, thr = 0.0f;
         const float E = err_per_norm * rnorm;
-        if (s1 + E <= stop_level) break;  // every exact score is below the stop level
-        const float thr = s1 - 2.0f * E;
+        const float win2 = 2.0f * err_per_norm * rnorm;
+        bool first = !PRUNE, done = false;
+        for (;;) {
+          for (int mc = 0; mc < M; mc += kChunk) {
+            const int mend = min(kChunk, M - mc);
+            // (a) one lane per atom: G_k = sum_j conj(d[j,k]) r[j,k]
+            for (int ml = lane; ml < mend; ml += 32) {
+              const int m = mc + ml;
+              float gv[GS];
+#pragma unroll
+              for (int q = 0; q < GS; ++q) gv[q] = 0.0f;
+              const float2 *dm = dT + m;
+              const float2 *r2 = reinterpret_cast<const float2 *>(s_rhi);
+#pragma unroll
+              for (int k = 0; k <= KM; ++k) {
+                if (k < H) {
+                  float gre0 = 0.f, gre1 = 0.f, gim0 = 0.f, gim1 = 0.f;
+#pragma unroll 2
+                  for (int j = 0; j < J; ++j, ++r2, dm += M) {
+                    const float2 dv = *dm, rv = *r2;
+                    gre0 = fmaf(dv.x, rv.x, gre0);
+                    gre1 = fmaf(dv.y, rv.y, gre1);
+                    gim0 = fmaf(dv.x, rv.y, gim0);
+                    gim1 = fmaf(-dv.y, rv.x, gim1);
+                  }
+                  if (k == 0) {
+                    gv[0] = gre0 + gre1;
+                  } else {
+                    gv[2 * k - 1] = 2.0f * (gre0 + gre1);
+                    gv[2 * k] = -2.0f * (gim0 + gim1);
+                  }
+                }
+              }
+              float4 *g4 = reinterpret_cast<float4 *>(s_g + ml * GS);
+#pragma unroll
+              for (int q = 0; q < GS / 4; ++q)
+                g4[q] = make_float4(gv[4 * q], gv[4 * q + 1], gv[4 * q + 2], gv[4 * q + 3]);
+              if constexpr (PRUNE) {
+                // |score(m, r)| <= |G_0| + 2 sum_k |G_k| for every angle
+                // (triangle inequality; gv holds G_0 and 2 Re / -2 Im of G_k),
+                // times a slack covering the FP32 rounding of this sum and of
+                // the transform below, so every FP32 score of the atom is <= ub
+                float ub = fabsf(gv[0]);
+#pragma unroll
+                for (int k = 1; k <= KM; ++k)
+                  if (k <= kmax) ub += sqrtf(fmaf(gv[2 * k - 1], gv[2 * k - 1], gv[2 * k] * gv[2 * k]));
+                s_ub[ml] = ub * (1.0f + 16.0f * (KM + 2) * 5.9604644775390625e-8f);
+              }
+            }
+            __syncwarp();
+            // (b) one lane per angle (or two): its value of every atom
+            auto scores = [&](int ml, float (&out)[NV]) {
+              const float4 *g4 = reinterpret_cast<const float4 *>(s_g + ml * GS);
+              float gv[GS];
+#pragma unroll
+              for (int q = 0; q < GS / 4; ++q) {
+                float4 v = g4[q];
+                gv[4 * q] = v.x;
+                gv[4 * q + 1] = v.y;
+                gv[4 * q + 2] = v.z;
+                gv[4 * q + 3] = v.w;
+              }
+#pragma unroll
+              for (int i = 0; i < RPL; ++i) {
+                // even harmonics (with k = 0) and odd ones, Re and Im terms apart
+                float s0[2] = {gv[0], 0.0f}, s2[2] = {0.0f, 0.0f};
+#pragma unroll
+                for (int k = 0; k < KM; ++k) {
+                  const int odd = (k + 1) & 1;
+                  s0[odd] = fmaf(gv[2 * k + 1], tc[i][k], s0[odd]);
+                  s2[odd] = fmaf(gv[2 * k + 2], ts[i][k], s2[odd]);
+                }
+                const float ev = s0[0] + s2[0], od = s0[1] + s2[1];
+                if constexpr (PAIR) {
+                  out[2 * i] = ev + od;
+                  out[2 * i + 1] = ev - od;
+                } else {
+                  out[i] = ev + od;
+                }
+              }
+            };
+            // (c) per-lane top-4
+            auto transform = [&](int ml) {
+              float out[NV];
+              scores(ml, out);
+#pragma unroll
+              for (int q = 0; q < NV; ++q) {
+                const float v = fabsf(out[q]);
+                // a value more than 2E below this lane's running best is below
+                // the final window and need not be kept (the best only grows)
+                if (valid(q) && !(v < tv[0] - win2))
+                  top4_insert(tv, ti, disc, v, (mc + ml) * R + r_of(q));
+              }
+            };
+            if (first) {
+#pragma unroll 1
+              for (int ml = 0; ml < mend; ++ml) {
+                float out[NV];
+                scores(ml, out);
+#pragma unroll
+                for (int q = 0; q < NV; ++q) {
+                  const float v = fabsf(out[q]);
+                  sv[q] = fmaxf(sv[q], fminf(v, bv[q]));
+                  bm[q] = v > bv[q] ? mc + ml : bm[q];
+                  bv[q] = fmaxf(bv[q], v);
+                }
+              }
+            } else           if constexpr (!PRUNE) {
+              for (int ml = 0; ml < mend; ++ml) transform(ml);
+            } else {
+              // In index order, an atom whose bound is below the warp's running
+              // best minus the window 2E (refreshed every 8 atoms; a stale best
+              // is lower, so only more atoms are transformed) is skipped: every
+              // FP32 score of it is below best - 2E <= the final threshold
+              // s1 - 2E (the best only grows), so none of them could be a
+              // candidate or raise a lane's discarded value to the threshold;
+              // the best atom is never skipped (its bound is >= its score).
+              // It rules out 52% of the transforms at M = 64, R = 64, K = 5, yet
+              // takes longer than the plain loop, whose unbroken run of short
+              // FMA chains pipelines better than a data-dependent skip.
+              float wbest = -INFINITY;
+              for (int ml = 0; ml < mend; ++ml) {
+                if ((ml & 7) == 0) wbest = warp_max(tv[0]);
+                if (s_ub[ml] < wbest - win2) continue;
+                transform(ml);
+              }
+            }
+            __syncwarp();
+          }
+          float top = tv[0];
+          if (first) {
+#pragma unroll
+            for (int q = 0; q < NV; ++q) {
+              if (!valid(q)) bv[q] = sv[q] = -INFINITY;
+              top = fmaxf(top, bv[q]);
+            }
+          }
+          s1 = warp_max(top);
+          if (s1 + E <= stop_level) {  // every exact score is below the stop level
+            done = true;
+            break;
+          }
+          thr = s1 - 2.0f * E;
+          if (!first) break;
+          bool close = false;
+#pragma unroll
+          for (int q = 0; q < NV; ++q) close |= sv[q] >= thr;
+          if (!__any_sync(0xffffffffu, close)) break;
+          first = false;
+        }
+        if (done) break;
         const bool overflow = __any_sync(0xffffffffu, disc >= thr);
 
         // ---- candidates, re-scored in double-float against the exact residual
         int ncand = 0;
-        if (!overflow) {
+        auto keep = [&](bool f, int c) {
+          const unsigned b = __ballot_sync(0xffffffffu, f);
+          if (f) s_cand[ncand + __popc(b & ((1u << lane) - 1u))] = c;
+          ncand += __popc(b);
+        };
+        if (first) {
 #pragma unroll
-          for (int q = 0; q < 4; ++q) {
-            const bool f = (tv[q] >= thr) && (ti[q] >= 0);
-            const unsigned b = __ballot_sync(0xffffffffu, f);
-            if (f) s_cand[ncand + __popc(b & ((1u << lane) - 1u))] = ti[q];
-            ncand += __popc(b);
-          }
+          for (int q = 0; q < NV; ++q) keep(bv[q] >= thr && bm[q] >= 0, bm[q] * R + r_of(q));
+        } else if (!overflow) {
+#pragma unroll
+          for (int q = 0; q < 4; ++q) keep(tv[q] >= thr && ti[q] >= 0, ti[q]);
         } else {
           if (lane == 0 && a.fallbacks) atomicAdd(a.fallbacks, 1ull);
           ncand = M * R;
@@ -393,8 +477,9 @@ __global__ void __launch_bounds__(256)
           const int c = overflow ? ci : s_cand[ci];
           const int m = c / R, r = c - m * R;
           df s = df_make(0.0f);
+#pragma unroll 1
           for (int e = lane; e < HJ; e += 32) {
-            const int k = e / J;
+            const int k = k_of(e);
             Cdf A = steered_entry(a.d, HJ, k, m, r, e, tw);
             df rr = {s_rhi[2 * e], s_rlo[2 * e]};
             df ri = {s_rhi[2 * e + 1], s_rlo[2 * e + 1]};
@@ -412,10 +497,11 @@ __global__ void __launch_bounds__(256)
 
       // ---- (e) new steered atom (cached), its Gram row, diagonal, right-hand side
       const int mn = best_c / R, rn = best_c - mn * R;
+      df sd = df_make(0.0f), sb = df_make(0.0f), sg = df_make(0.0f);
       {
-        df sd = df_make(0.0f), sb = df_make(0.0f);
+#pragma unroll 1
         for (int e = lane; e < HJ; e += 32) {
-          const int k = e / J;
+          const int k = k_of(e);
           Cdf A = steered_entry(a.d, HJ, k, mn, rn, e, tw);
           s_A[t * HJ + e] = cdf_pack(A);
           df qd = df_add(df_mul(A.re, A.re), df_mul(A.im, A.im));
@@ -425,14 +511,12 @@ __global__ void __launch_bounds__(256)
         }
         sd = df_warp_sum(sd);
         sb = df_warp_sum(sb);
-        if (lane == 0) {
-          s_gram[t] = df_to_d(sd);
-          s_gram[t + 1] = df_to_d(sb);
-        }
       }
       __syncwarp();
+#pragma unroll 1
       for (int i = 0; i < t; ++i) {
         df s = df_make(0.0f);
+#pragma unroll 1
         for (int e = lane; e < HJ; e += 32) {
           const Cdf A = cdf_unpack(s_A[t * HJ + e]);
           const Cdf B = cdf_unpack(s_A[i * HJ + e]);
@@ -440,54 +524,55 @@ __global__ void __launch_bounds__(256)
           s = df_add(s, (e >= J) ? df_mul_f(q, 2.0f) : q);
         }
         s = df_warp_sum(s);
-        if (lane == 0) s_gram[K + 1 + i] = df_to_d(s);  // Gram row, after diag/rhs slots
+        if (lane == i) sg = s;
       }
-      __syncwarp();
-      int ok = 0;
+      // New row t of L (packed lower triangle, row i starts at i(i+1)/2) and the
+      // solve of all t + 1 weights in FP64, lane i holding entry i: an FP64
+      // instruction takes the pipe for 64 cycles however many lanes take part.
+      const double diag = df_to_d(sd);
+      double p2 = diag, zt = df_to_d(sb), g = df_to_d(sg), lrow = 0.0;
+#pragma unroll 1
+      for (int j = 0; j < t; ++j) {
+        const double lj = __shfl_sync(0xffffffffu, g * s_inv[j], j);
+        if (lane == j) lrow = lj;
+        if (lane > j && lane < t) g -= s_L[lane * (lane + 1) / 2 + j] * lj;
+        p2 -= lj * lj;
+        zt -= lj * s_z[j];
+      }
+      if (!(p2 > kPivotRel * diag)) break;
+      const double inv = rsqrt(p2);  // 1 / L_tt (L_tt itself is not needed)
+      zt *= inv;
+      if (lane < t) s_L[t * (t + 1) / 2 + lane] = lrow;
       if (lane == 0) {
-        // new row t of L (packed lower triangle, row i starts at i(i+1)/2); FP64
-        const double diag = s_gram[t], rhs = s_gram[t + 1];
-        double *Lt = s_L + t * (t + 1) / 2;
-        double p2 = diag;
-        for (int i = 0; i < t; ++i) {
-          const double *Li = s_L + i * (i + 1) / 2;
-          double v = s_gram[K + 1 + i];
-          for (int j = 0; j < i; ++j) v -= Li[j] * Lt[j];
-          v *= s_inv[i];
-          Lt[i] = v;
-          p2 -= v * v;
-        }
-        if (p2 > kPivotRel * diag) {
-          ok = 1;
-          const double ltt = sqrt(p2);
-          Lt[t] = ltt;
-          s_inv[t] = 1.0 / ltt;
-          double zt = rhs;
-          for (int i = 0; i < t; ++i) zt -= Lt[i] * s_z[i];
-          s_z[t] = zt * s_inv[t];
-          // back substitution L^T a = z over the t+1 selected atoms
-          for (int i = t; i >= 0; --i) {
-            double v = s_z[i];
-            for (int q = i + 1; q <= t; ++q) v -= s_L[q * (q + 1) / 2 + i] * s_a[q];
-            v *= s_inv[i];
-            s_a[i] = v;
-            const float hi = __double2float_rn(v);
-            s_adf[2 * i] = hi;
-            s_adf[2 * i + 1] = __double2float_rn(v - (double)hi);
-          }
-          s_sel[t] = best_c;
-        }
+        s_inv[t] = inv;
+        s_z[t] = zt;
+        s_sel[t] = best_c;
       }
-      ok = __shfl_sync(0xffffffffu, ok, 0);
       __syncwarp();
-      if (!ok) break;
+      // back substitution L^T a = z
+      double w = lane <= t ? s_z[lane] : 0.0, coef = 0.0;
+#pragma unroll 1
+      for (int i = t; i >= 0; --i) {
+        const double ai = __shfl_sync(0xffffffffu, w * s_inv[i], i);
+        if (lane == i) coef = ai;
+        if (lane < i) w -= s_L[i * (i + 1) / 2 + lane] * ai;
+      }
+      if (lane <= t) {
+        s_a[lane] = coef;
+        const float hi = __double2float_rn(coef);
+        s_adf[2 * lane] = hi;
+        s_adf[2 * lane + 1] = __double2float_rn(coef - (double)hi);
+      }
+      __syncwarp();
       ++t;
 
       // ---- (d) residual x - sum_i a_i S_{r_i} d_{m_i} (double-float)
       df nacc = df_make(0.0f);
+#pragma unroll 1
       for (int e = lane; e < HJ; e += 32) {
         df rr = df_make(s_x[2 * e]);
         df ri = df_make(s_x[2 * e + 1]);
+#pragma unroll 1
         for (int i = 0; i < t; ++i) {
           const Cdf A = cdf_unpack(s_A[i * HJ + e]);
           const df ai = {s_adf[2 * i], s_adf[2 * i + 1]};
@@ -530,7 +615,7 @@ __global__ void __launch_bounds__(256)
   }
 }
 
-template <int KM, int RPL, bool PRUNE>
+template <int KM, int RPL, bool PAIR, bool PRUNE>
 int launch_p(const RompArgs &a, cudaStream_t stream) {
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
@@ -540,7 +625,8 @@ int launch_p(const RompArgs &a, cudaStream_t stream) {
   cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
   const int HJ = a.H * a.J;
   bool dT_smem = (size_t)2 * HJ * a.M * 4 <= 64 * 1024;
-  int warps = 8;
+  // few patches: smaller blocks, over more SMs
+  int warps = a.redo_list || a.P <= (int64_t)16 * nsm ? 8 : BlockWarps<KM, RPL, PRUNE>::v;
   Layout L = make_layout<KM>(a.M, a.J, a.H, a.R, a.K, warps, dT_smem);
   while (L.total > max_optin && warps > 1) {
     warps >>= 1;
@@ -556,7 +642,7 @@ int launch_p(const RompArgs &a, cudaStream_t stream) {
     }
   }
   if (L.total > max_optin) return RSC_ERR_UNSUPPORTED;
-  auto kern = romp_f32_kernel<KM, RPL, PRUNE>;
+  auto kern = romp_f32_kernel<KM, RPL, PAIR, PRUNE>;
   e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, L.total);
   if (e != cudaSuccess) return rsc_cuda_fail(e);
   int per_sm = 0;
@@ -574,25 +660,32 @@ int launch_p(const RompArgs &a, cudaStream_t stream) {
   return RSC_OK;
 }
 
-template <int KM, int RPL>
+template <int KM, int RPL, bool PAIR>
 int launch_t(const RompArgs &a, cudaStream_t stream) {
-  return a.prune ? launch_p<KM, RPL, true>(a, stream) : launch_p<KM, RPL, false>(a, stream);
+  return a.prune ? launch_p<KM, RPL, PAIR, true>(a, stream)
+                 : launch_p<KM, RPL, PAIR, false>(a, stream);
+}
+
+template <int KM>
+int launch_k(const RompArgs &a, cudaStream_t stream) {
+  // (harmonics above 12: angles up to 64 only, as their factors fill the registers)
+  if (a.R % 2 == 0) {
+    if (a.R <= 64) return launch_t<KM, 1, true>(a, stream);
+    if constexpr (KM <= 12) return launch_t<KM, 2, true>(a, stream);
+  } else {
+    if (a.R <= 64) return launch_t<KM, 2, false>(a, stream);
+    if constexpr (KM <= 12) return launch_t<KM, 4, false>(a, stream);
+  }
+  return RSC_ERR_UNSUPPORTED;
 }
 
 }  // namespace
 
 int rsc_launch_f32(const RompArgs &a, cudaStream_t stream) {
   if (a.P == 0) return RSC_OK;
-  const int rpl = (a.R + 31) / 32;
-  if (a.kmax <= 8) {
-    if (rpl == 1) return launch_t<8, 1>(a, stream);
-    if (rpl == 2) return launch_t<8, 2>(a, stream);
-    if (rpl <= 4) return launch_t<8, 4>(a, stream);
-  } else if (a.kmax <= 12) {
-    if (rpl <= 2) return launch_t<12, 2>(a, stream);
-    if (rpl <= 4) return launch_t<12, 4>(a, stream);
-  } else if (a.kmax <= 16) {
-    if (rpl <= 2) return launch_t<16, 2>(a, stream);
-  }
+  if (a.R > kMaxR) return RSC_ERR_UNSUPPORTED;
+  if (a.kmax <= 8) return launch_k<8>(a, stream);
+  if (a.kmax <= 12) return launch_k<12>(a, stream);
+  if (a.kmax <= 16) return launch_k<16>(a, stream);
   return RSC_ERR_UNSUPPORTED;
 }

@@ -745,8 +745,8 @@ int rsc_dict_create(const float *coef, rsc_dims dims, void *stream, rsc_dict **o
   std::vector<float> hT((size_t)2 * HJ * M);
   for (int m = 0; m < M; ++m)
     for (int q = 0; q < HJ; ++q) {
-      hT[(size_t)q * M + m] = h[((size_t)m * HJ + q) * 2];
-      hT[(size_t)(HJ + q) * M + m] = h[((size_t)m * HJ + q) * 2 + 1];
+      hT[((size_t)q * M + m) * 2] = h[((size_t)m * HJ + q) * 2];
+      hT[((size_t)q * M + m) * 2 + 1] = h[((size_t)m * HJ + q) * 2 + 1];
     }
   // steering factors exp(-i k 2 pi r / R) of Eq. (Sr) as cos/sin in
   // double-float (hi + lo) from FP64, argument reduced exactly: k r mod R

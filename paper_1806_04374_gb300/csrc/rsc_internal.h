@@ -22,7 +22,7 @@ struct rsc_dict {
   int M, J, kmax, R, H;  // H = kmax + 1
   int device;
   float *d;      // [M][H][J][2]  atoms as given
-  float *dT;     // [2][H*J][M]   re plane, im plane: lane-per-atom reads
+  float *dT;     // [H*J][M]      (re, im): lane-per-atom reads
   float *tw;     // [4][H][R]     cos hi, cos lo, sin hi, sin lo of 2 pi k r / R
   int *err;      // device error word (first error code recorded)
   unsigned long long *fallbacks;  // device counter of exact re-scans
