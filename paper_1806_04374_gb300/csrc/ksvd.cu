@@ -36,7 +36,10 @@
 namespace {
 
 constexpr int kCovThreads = 384;  // one 4 x 4 tile each: all 351 tiles of n = 102 in one round
-constexpr int kFillChunk = 256;   // patches per chunk of the sample lists
+// patches per chunk of the sample lists: 1,563 blocks at 200,000 patches, so that
+// the last of them leave few SMs idle (256 patches 0.39 ms, 128 0.33, 64 0.31, but
+// a count per chunk and atom to scan)
+constexpr int kFillChunk = 128;
 constexpr int kMaxAtomsKsvd = 12288;  // per-atom cursors of a chunk in shared memory
 constexpr int kCovBatch = 32;
 constexpr int kEigThreads = 256;
@@ -169,24 +172,47 @@ __global__ void __launch_bounds__(256) ksvd_offset_kernel(const KsvdArgs a) {
 }
 
 // Per chunk: the residuals e_p = x_p - sum_i a_i S_{r_i} d_{m_i} of its
-// patches in double-float with their coding errors, a warp per patch (lanes
-// over the entries: a thread per patch read 32 rows with every load, 0.93 ms
-// per 200,000 patches at K = 5), and the chunk's sample slots in patch order:
-// 32 occurrences at a time in order, those of the same atom ranked by a match
-// over the warp, so every atom's list is in patch order on every run.
+// patches in double-float with their coding errors, a warp per patch, and the
+// chunk's sample slots in patch order: warp 0 takes 32 occurrences at a time in
+// order, those of the same atom ranked by a match over the warp, so every
+// atom's list is in patch order on every run.
+//
+// Bound by the double-float arithmetic: 0.33 ms per 200,000 patches at K = 5 and
+// n = 102 (0.93 with a thread per patch, which read 32 rows with every load;
+// 0.45 with patches dealt to the warps, the seven others waiting for warp 0).
 constexpr int kFillThreads = 256;
 
+__device__ __forceinline__ unsigned char *smem_align16(unsigned char *p) {
+  return reinterpret_cast<unsigned char *>((reinterpret_cast<uintptr_t>(p) + 15) & ~uintptr_t(15));
+}
+
+template <bool TW>
 __global__ void __launch_bounds__(kFillThreads) ksvd_fill_kernel(const KsvdArgs a) {
   // [kFillChunk][K] code (weight hi, lo, atom or -1, angle); [M] next slot of
   // each atom in this chunk; [kFillChunk][K] slot of each chosen occurrence
   extern __shared__ __align__(16) int4 s_code[];
   const int J = a.J, H = a.H, HJ = H * J, R = a.R, K = a.K;
   int *cur = reinterpret_cast<int *>(s_code + kFillChunk * K), *slot = cur + a.M;
+  // the steering factors as [R][H] (cos hi, lo, sin hi, lo) where they fit: one
+  // load of 16 bytes in place of four in different lines
+  float4 *s_tw = reinterpret_cast<float4 *>(
+      smem_align16(reinterpret_cast<unsigned char *>(slot + kFillChunk * K)));
+  __shared__ int s_next;
+  if (threadIdx.x == 0) s_next = 0;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int64_t p0 = (int64_t)blockIdx.x * kFillChunk;
   const int np = (int)min((int64_t)kFillChunk, a.P - p0);
   for (int m = threadIdx.x; m < a.M; m += kFillThreads)
     cur[m] = a.offset[m] + a.chunk_base[(size_t)blockIdx.x * a.M + m];
+  auto factors = [&](int k, int r) {
+    return make_float4(a.tw[(0 * H + k) * R + r], a.tw[(1 * H + k) * R + r],
+                       a.tw[(2 * H + k) * R + r], a.tw[(3 * H + k) * R + r]);
+  };
+  if (TW)
+    for (int i = threadIdx.x; i < R * H; i += kFillThreads) {
+      const int k = i / R, r = i - k * R;
+      s_tw[r * H + k] = factors(k, r);
+    }
   for (int i = threadIdx.x; i < np * K; i += kFillThreads) {
     const df w = df_from_d(a.coef[p0 * K + i]);
     s_code[i] = make_int4(__float_as_int(w.hi), __float_as_int(w.lo), a.atom[p0 * K + i],
@@ -206,7 +232,12 @@ __global__ void __launch_bounds__(kFillThreads) ksvd_fill_kernel(const KsvdArgs 
     }
   }
   const df sqrt2 = df_from_d(1.4142135623730951);
-  for (int pl = warp; pl < np; pl += kFillThreads / 32) {
+  // (patches are drawn, not dealt: warp 0 comes later)
+  for (;;) {
+    int pl = 0;
+    if (lane == 0) pl = atomicAdd(&s_next, 1);
+    pl = __shfl_sync(0xffffffffu, pl, 0);
+    if (pl >= np) break;
     const int64_t p = p0 + pl;
     df n2 = df_make(0.0f);
     for (int e = lane; e < HJ; e += 32) {
@@ -216,10 +247,9 @@ __global__ void __launch_bounds__(kFillThreads) ksvd_fill_kernel(const KsvdArgs 
       for (int i = 0; i < K; ++i) {
         const int4 c4 = s_code[pl * K + i];
         if (c4.z < 0) continue;
-        const int r = c4.w;
-        const df c = {a.tw[(0 * H + k) * R + r], a.tw[(1 * H + k) * R + r]};
-        const df sn = {a.tw[(2 * H + k) * R + r], a.tw[(3 * H + k) * R + r]};
-        const float2 dv = reinterpret_cast<const float2 *>(a.d)[(size_t)c4.z * HJ + e];
+        const float4 f = TW ? s_tw[c4.w * H + k] : factors(k, c4.w);
+        const df c = {f.x, f.y}, sn = {f.z, f.w};
+        const float2 dv = __ldg(reinterpret_cast<const float2 *>(a.d) + (size_t)c4.z * HJ + e);
         const float dim = k ? dv.y : 0.0f;
         const df w = {__int_as_float(c4.x), __int_as_float(c4.y)};
         // S_r d: harmonic k times exp(-i k theta_r)
@@ -411,7 +441,7 @@ __global__ void __launch_bounds__(kCovThreads) ksvd_cov_kernel(const KsvdArgs a)
 // Rows hold the real parts of the entries first, then the imaginary parts of
 // k >= 1, so that neighbouring lanes store to neighbouring rows.
 // 200,000 patches, K = 5, M = 128, n = 102, R = 64 (10^6 samples): 1.10 ms, and
-// the whole accumulation and update 1.77 ms (6.86 ms with every covariance on
+// the whole accumulation and update 1.67 ms (6.86 ms with every covariance on
 // the CUDA cores); C off by 1.8e-15 of its norm, 1.9e-15 there.
 // Every wait is bounded.
 constexpr int kTcvBuild = 15, kTcvSum = 8;  // warps
@@ -1174,13 +1204,16 @@ int ksvd_accumulate(KsvdArgs &a, cudaStream_t st) {
   a.state = tensor ? reinterpret_cast<int *>(take(bSt)) : nullptr;
   a.expo = tensor ? reinterpret_cast<int *>(take(bEx)) : nullptr;
   const size_t hist_smem = (size_t)M * 4;
-  const size_t fill_smem = (size_t)kFillChunk * a.K * 20 + hist_smem;
+  const bool fill_tw = (size_t)a.R * a.H * 16 <= kTcvTwMax;
+  const size_t fill_smem =
+      (size_t)kFillChunk * a.K * 20 + hist_smem + (fill_tw ? (size_t)a.R * a.H * 16 + 16 : 0);
+  auto fill = fill_tw ? ksvd_fill_kernel<true> : ksvd_fill_kernel<false>;
   const size_t cov_smem = (size_t)2 * kCovBatch * (4 * ((n + 3) / 4) + 4) * 4;
   const size_t tc_smem = kTcvTwOff + (size_t)a.R * a.H * 16 + 1024;
   e = cudaFuncSetAttribute(ksvd_cov_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                            (int)cov_smem);
   if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(ksvd_fill_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    e = cudaFuncSetAttribute(fill, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)fill_smem);
   if (e == cudaSuccess && tensor)
     e = cudaFuncSetAttribute(ksvd_cov_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -1189,7 +1222,7 @@ int ksvd_accumulate(KsvdArgs &a, cudaStream_t st) {
     ksvd_chunk_count_kernel<<<a.nchunk, 256, hist_smem, st>>>(a);
     ksvd_atom_scan_kernel<<<M, 256, 0, st>>>(a);
     ksvd_offset_kernel<<<1, 256, 0, st>>>(a);
-    ksvd_fill_kernel<<<a.nchunk, kFillThreads, fill_smem, st>>>(a);
+    fill<<<a.nchunk, kFillThreads, fill_smem, st>>>(a);
     if (tensor) ksvd_cov_tc_kernel<<<M * a.split, kTcvThreads, tc_smem, st>>>(a, (n + 15) / 16 * 16);
     ksvd_cov_kernel<<<M * a.split, kCovThreads, cov_smem, st>>>(a);
     const size_t work = tensor ? (size_t)M * kTcvPlaces : (size_t)M * n * n;
