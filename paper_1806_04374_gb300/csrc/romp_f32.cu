@@ -629,7 +629,7 @@ int launch_p(const RompArgs &a, cudaStream_t stream) {
   int warps = a.redo_list || a.P <= (int64_t)16 * nsm ? 8 : BlockWarps<KM, RPL, PRUNE>::v;
   Layout L = make_layout<KM>(a.M, a.J, a.H, a.R, a.K, warps, dT_smem);
   while (L.total > max_optin && warps > 1) {
-    warps >>= 1;
+    warps = warps > 8 ? warps - 1 : warps >> 1;
     L = make_layout<KM>(a.M, a.J, a.H, a.R, a.K, warps, dT_smem);
   }
   if (L.total > max_optin && dT_smem) {

@@ -32,6 +32,7 @@ CASES = [
     ("kmax0_long", 40, 300, 0, 1, 4, 20, 1),
     ("K16", 40, 6, 8, 32, 16, 40, 1),
     ("many_patches", 8, 6, 8, 32, 3, 2600, 1),
+    ("many_patches_K16", 40, 6, 8, 32, 16, 2600, 1),
     ("twins", 40, 6, 8, 64, 4, 40, 2),
     ("twins_odd_R", 40, 6, 8, 33, 4, 40, 2),
     ("six_copies", 48, 6, 8, 64, 3, 40, 6),
