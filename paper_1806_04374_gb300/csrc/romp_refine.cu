@@ -33,6 +33,8 @@
 // 432 bytes, M = R = 64, K = 5, that kept the L1 tag stage busy for
 // 1.06 ms per step (10,000 cycles per warp and step, DRAM at 16%), while
 // these loads touch the 4 lines of one row.
+#include <algorithm>
+
 #include "rsc_internal.h"
 #include "tc_common.cuh"
 
@@ -257,14 +259,15 @@ __global__ void __launch_bounds__(128) romp_init_kernel(const RefineArgs a) {
   const StateIdx I(a.K);
   const int lane = threadIdx.x & 31, vec = 2 * a.H * a.J;
   const LaneSlots<LAY> ls(lane, a.J, a.kmax);
-  const int64_t P = a.P, step = (int64_t)gridDim.x * blockDim.x;
-  for (int64_t base = (int64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31); base < P;
-       base += step) {
+  const int64_t P = a.P, step = (int64_t)gridDim.x * (blockDim.x >> 5) * a.warp_patches;
+  for (int64_t base = ((int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * a.warp_patches;
+       base < P; base += step) {
     const int64_t p = base + lane;
     float xnorm = 0.0f, n2 = 0.0f;
     df x2 = df_make(0.0f);
     int e = 0;
-    unsigned todo = __ballot_sync(0xffffffffu, p < P);
+    const bool mine = lane < a.warp_patches && p < P;
+    unsigned todo = __ballot_sync(0xffffffffu, mine);
     while (todo) {
       int src[B], slot;
       next_batch<B>(todo, lane, src, slot);
@@ -300,7 +303,7 @@ __global__ void __launch_bounds__(128) romp_init_kernel(const RefineArgs a) {
         e = er;
       }
     }
-    if (p < P) {
+    if (mine) {
       const float rn = sqrtf(n2), dr = residual_err(0, xnorm, 0.0f);
       a.sI[I.iE * P + p] = e;
       a.sF[I.fX * P + p] = xnorm;
@@ -319,8 +322,8 @@ __global__ void __launch_bounds__(128) romp_init_kernel(const RefineArgs a) {
 // 10^6 patches, M = R = 64, K = 5: 0.69 ms per step on average (0.62 / 0.81 /
 // 0.98 at T = 1 / 2 / 3) against 1.06 for a thread per patch; the call 9.00 ->
 // 7.29 ms, 1,000 patches at M = 16 261 -> 129 us (one kernel per step, not a
-// memset and two passes), the 21 x 21 image sizes 21.8 -> 16.3 ms.  Issue is
-// at 50%, so both instructions (12,000 to 17,000 per warp) and the loads'
+// memset and two passes; 81 with fewer patches a warp, see the launch), the
+// 21 x 21 image sizes 21.8 -> 16.3 ms.  Issue is at 50%, so both instructions (12,000 to 17,000 per warp) and the loads'
 // latency count.  Registers: at most 128 (4 blocks an SM) 3.79 ms per call of
 // init and refines; without a cap (up to 255) 4.24, 5 or 6 blocks 3.96 / 3.91
 // (spills).
@@ -335,11 +338,11 @@ __global__ void __launch_bounds__(128, 4) romp_refine_kernel(const RefineArgs a)
   const int R = a.R, M = a.M, Rr = a.Rr;
   const LaneSlots<LAY> ls(lane, a.J, a.kmax);
   const TwS tw{a.tw, a.H, R};  // only for Gram entries without a table
-  const int64_t P = a.P, step = (int64_t)gridDim.x * blockDim.x;
-  for (int64_t base = (int64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31); base < P;
-       base += step) {
+  const int64_t P = a.P, step = (int64_t)gridDim.x * (blockDim.x >> 5) * a.warp_patches;
+  for (int64_t base = ((int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * a.warp_patches;
+       base < P; base += step) {
     const int64_t p = base + lane;
-    const bool act = p < P && a.status[p] > 0;
+    const bool act = lane < a.warp_patches && p < P && a.status[p] > 0;
     if (!__any_sync(0xffffffffu, act)) continue;
     Ls<T + 1> S;
     int e = 0;
@@ -727,10 +730,17 @@ int rsc_launch_refine(const RefineArgs &a, int step, cudaStream_t stream) {
   const cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return rsc_cuda_fail(e);
   cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-  const int64_t blocks = (a.P + 127) / 128;
+  // A warp takes 32 patches, or fewer (whole batches of rows, the other lanes
+  // idle in the scalar parts) while that still leaves the SMs' 16 warps each
+  // with work: a small call is one warp's chain of batches long.  1,000 patches
+  // at M = 16, R = 32, K = 3: 127 us a call with 32 patches a warp, 81 with 4.
+  RefineArgs w = a;
+  const int64_t share = (a.P + 16 * nsm - 1) / (16 * nsm);
+  w.warp_patches = (int)std::min<int64_t>(32, (share + 3) / 4 * 4);
+  const int64_t per_block = 4 * w.warp_patches, blocks = (a.P + per_block - 1) / per_block;
   const int64_t cap = (int64_t)nsm * (a.blocks_per_sm > 0 ? a.blocks_per_sm : 32);
   const unsigned grid = (unsigned)(blocks < cap ? blocks : cap);
-  if (a.L == kTcKstLong) return launch_refine_l<kLong>(a, step, grid, stream);
-  return a.paired ? launch_refine_l<kPaired>(a, step, grid, stream)
-                  : launch_refine_l<kPlain>(a, step, grid, stream);
+  if (a.L == kTcKstLong) return launch_refine_l<kLong>(w, step, grid, stream);
+  return a.paired ? launch_refine_l<kPaired>(w, step, grid, stream)
+                  : launch_refine_l<kPlain>(w, step, grid, stream);
 }

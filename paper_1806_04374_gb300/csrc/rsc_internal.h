@@ -249,6 +249,7 @@ struct RefineArgs {
   const unsigned *cand_mask;  // see ScoreArgs
   float *win;            // [P] window of the next scoring pass (see ScoreArgs)
   int paired;            // rows and candidates in the paired layout (rsc_slot_code)
+  int warp_patches;      // patches of a warp (set by the launch)
   int *status;           // 1 active, 0 done, -1 handed to the FP32 path
   double *sD;            // state, structure of arrays
   float *sF;

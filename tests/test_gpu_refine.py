@@ -48,3 +48,20 @@ def test_layout_edges(rsc, case):
     g = run_gpu(rsc, x, d, R, K, "f16")
     x[:, 0, :, 1] = 0.0
     check(x, d, R, K, g, TOL)
+
+
+@pytest.mark.parametrize("J,kmax,R", [(6, 8, 32), (6, 8, 33), (10, 12, 16)],
+                         ids=["paired", "plain", "long"])
+def test_patches_of_a_warp(rsc, J, kmax, R):
+    """32 patches a warp, or 4 to 28 in small calls: the same bits."""
+    import torch
+    d = synth.make_dictionary(9, J, kmax, 77)
+    x, _ = synth.make_patches(d, 80_000, 3, 0.1, 78)
+    dic = rsc.Dictionary(torch.from_numpy(d).cuda(), R)
+    xd = torch.from_numpy(x).cuda()
+    whole = rsc.encode(dic, xd, 3, "f16")
+    for lo, hi in ((0, 1), (1, 1000), (1000, 13_200), (13_200, 80_000)):
+        part = rsc.encode(dic, xd[lo:hi].contiguous(), 3, "f16")
+        for k, v in part.items():
+            assert torch.equal(v, whole[k][lo:hi]), (k, lo)
+    dic.close()
