@@ -422,7 +422,7 @@ def measure_projection(rsc, torch, dev, stream, reps: int = 5) -> dict:
 
 def measure_roundtrip(rsc, torch, dev, stream, dic, codes, reps: int = 5) -> dict:
     """The way back on the benchmark's own codes (10^6 patches, M = 64,
-    R = 64, K = 5): rsc_reconstruct (sum_i a_i S_i d_i, FP64 accumulation)
+    R = 64, K = 5): rsc_reconstruct (sum_i a_i S_i d_i, double-float)
     and rsc_synthesize (Phi x_hat on the 11 x 11 basis, 97 pixels), patches/s
     of each from CUDA events on the launching stream."""
     N, J, kmax = 11, 6, 8
