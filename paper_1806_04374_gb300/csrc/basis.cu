@@ -25,6 +25,7 @@
 // its image) and multiplies it by the analysis operator, writing half
 // spectra in the layout rsc_encode takes.
 #include <math.h>
+#include <stdint.h>
 #include <string.h>
 
 #include <algorithm>
@@ -327,9 +328,10 @@ __device__ __forceinline__ int find_item(const ImageItem *items, int n_items, in
   return lo;
 }
 
-// Top-left pixel of window p (null past the end) and its image's width.
-// `one`: the whole tile p0 .. last lies in one image (the same answer for
-// every thread of the tile).
+// Top-left pixel of window p (past the end: of the last one) and its image's width.
+// `one`: the whole tile p0 .. last lies in one image whose windows' pixel
+// offsets, up to (N - 1) w + N - 1, fit the 32 bits of the offset tables (the
+// same answer for every thread of the tile).
 __device__ __forceinline__ const float *find_window(const ImageItem *items, int n_items, int N,
                                                     int64_t p0, int64_t last, int64_t p, int &w,
                                                     bool &one) {
@@ -338,6 +340,7 @@ __device__ __forceinline__ const float *find_window(const ImageItem *items, int 
   if (p > last) p = last;
   if (!one) it = find_item(items, n_items, p);
   const ImageItem im = items[it];
+  one = one && (int64_t)(N - 1) * im.w + N - 1 <= INT32_MAX;
   const int64_t local = p - im.first;
   const int nw = im.w - N + 1;
   int r0, c0;
@@ -353,7 +356,7 @@ __device__ __forceinline__ const float *find_window(const ImageItem *items, int 
 }
 
 // Offsets of a window's pixels: from the group's table (a tile inside one
-// image) or from the mask and the thread's own image width.  Pixels past npix
+// image, see find_window) or from the mask and the thread's own image width.  Pixels past npix
 // read the mask's first one.
 struct PixelOffsets {
   const int *tab;
