@@ -924,8 +924,7 @@ int launch_project(const rsc_basis *b, const ImageItem *items_dev, int n_items, 
         project_tc_kernel<1>, project_tc_kernel<2>, project_tc_kernel<3>, project_tc_kernel<4>,
         project_tc_kernel<5>, project_tc_kernel<6>, project_tc_kernel<7>, project_tc_kernel<8>};
     const auto kern = kernels[b->KP / 16 - 1];
-    cudaError_t e =
-        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, total);
+    cudaError_t e = rsc_allow_smem(kern, (size_t)total);
     if (e != cudaSuccess) return rsc_cuda_fail(e);
     const int64_t tile_pairs = ((P_total + kPjRows - 1) / kPjRows + 1) / 2;
     const unsigned grid = (unsigned)std::min<int64_t>(tile_pairs, (int64_t)nsm);
@@ -935,8 +934,7 @@ int launch_project(const rsc_basis *b, const ImageItem *items_dev, int n_items, 
     return e == cudaSuccess ? RSC_OK : rsc_cuda_fail(e);
   }
   if (b->Bw) {
-    cudaError_t e = cudaFuncSetAttribute(project_tcw_kernel,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, kPwSmem);
+    cudaError_t e = rsc_allow_smem(project_tcw_kernel, (size_t)kPwSmem);
     if (e != cudaSuccess) return rsc_cuda_fail(e);
     const int64_t tiles = (P_total + 127) / 128;
     const unsigned grid = (unsigned)std::min<int64_t>(tiles, (int64_t)nsm);
@@ -948,8 +946,7 @@ int launch_project(const rsc_basis *b, const ImageItem *items_dev, int n_items, 
   }
   const int64_t blocks = (P_total + 127) / 128;
   const int shm = b->npix * 64 * (int)sizeof(float);
-  cudaError_t e =
-      cudaFuncSetAttribute(project_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, shm);
+  cudaError_t e = rsc_allow_smem(project_kernel, (size_t)shm);
   if (e != cudaSuccess) return rsc_cuda_fail(e);
   const int per_sm = std::max(1, std::min(4, (220 * 1024) / shm));  // by shared memory, registers
   const unsigned grid = (unsigned)std::min<int64_t>(blocks, (int64_t)nsm * per_sm);

@@ -1222,14 +1222,9 @@ int ksvd_accumulate(KsvdArgs &a, cudaStream_t st) {
   auto fill = fill_tw ? ksvd_fill_kernel<true> : ksvd_fill_kernel<false>;
   const size_t cov_smem = (size_t)2 * kCovBatch * (4 * ((n + 3) / 4) + 4) * 4;
   const size_t tc_smem = kTcvTwOff + (size_t)a.R * a.H * 16 + 1024;
-  e = cudaFuncSetAttribute(ksvd_cov_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           (int)cov_smem);
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(fill, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)fill_smem);
-  if (e == cudaSuccess && tensor)
-    e = cudaFuncSetAttribute(ksvd_cov_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)tc_smem);
+  e = rsc_allow_smem(ksvd_cov_kernel, cov_smem);
+  if (e == cudaSuccess) e = rsc_allow_smem(fill, fill_smem);
+  if (e == cudaSuccess && tensor) e = rsc_allow_smem(ksvd_cov_tc_kernel, tc_smem);
   if (e == cudaSuccess) {
     ksvd_chunk_count_kernel<<<a.nchunk, 256, hist_smem, st>>>(a);
     ksvd_atom_scan_kernel<<<M, 256, 0, st>>>(a);
@@ -1256,8 +1251,7 @@ int ksvd_accumulate(KsvdArgs &a, cudaStream_t st) {
 int ksvd_finish(KsvdArgs &a, cudaStream_t st) {
   const int n = a.n;
   const size_t eig_smem = ((size_t)n * n + 2 * n + 32) * 8;
-  cudaError_t e = cudaFuncSetAttribute(ksvd_eig_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)eig_smem);
+  cudaError_t e = rsc_allow_smem(ksvd_eig_kernel, eig_smem);
   if (e == cudaSuccess) {
     ksvd_eig_kernel<<<a.M, kEigThreads, eig_smem, st>>>(a, 5000);
     ksvd_reset_kernel<<<1, 256, 0, st>>>(a);

@@ -240,7 +240,7 @@ cudaError_t launch_reconstruct(const rsc_dict *dict, int dev, int64_t P, int K, 
   if (PAIRS) per = (per + 1) & ~1;
   const size_t smem = (size_t)R * H * 16 + (size_t)nw * tile * K * 16;
   auto kern = reconstruct_kernel<PAIRS>;
-  e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  e = rsc_allow_smem(kern, smem);
   int per_sm = 0;
   if (e == cudaSuccess)
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kRecThreads, smem);
@@ -418,8 +418,7 @@ cudaError_t launch_synthesize(const rsc_basis_view &v, int dev, int64_t P, const
     if ((v.nout + c - 1) / c * c < (v.nout + kc - 1) / kc * kc) kc = c;
   const size_t smem = std::max((size_t)2 * kc * (BM + 8 * ct), (size_t)BM * 8 * ct) * 4;
   auto kern = synthesize_kernel<RT>;
-  cudaError_t e =
-      cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = rsc_allow_smem(kern, smem);
   int nsm = 0, per_sm = 0;
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
   if (e == cudaSuccess)

@@ -643,7 +643,7 @@ int launch_p(const RompArgs &a, cudaStream_t stream) {
   }
   if (L.total > max_optin) return RSC_ERR_UNSUPPORTED;
   auto kern = romp_f32_kernel<KM, RPL, PAIR, PRUNE>;
-  e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, L.total);
+  e = rsc_allow_smem(kern, (size_t)L.total);
   if (e != cudaSuccess) return rsc_cuda_fail(e);
   int per_sm = 0;
   e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, warps * 32, L.total);

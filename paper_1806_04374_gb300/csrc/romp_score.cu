@@ -423,7 +423,7 @@ int launch_score_t(const ScoreArgs &a, const CUtensorMap &tmA, const CUtensorMap
   constexpr int total = SShape<PAIRED, NB, STAGES>::total;
   if (total > max_optin) return RSC_ERR_UNSUPPORTED;
   auto kern = romp_score_kernel<PAIRED, NB, STAGES>;
-  e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, total);
+  e = rsc_allow_smem(kern, (size_t)total);
   if (e != cudaSuccess) return rsc_cuda_fail(e);
   const int64_t tiles = (a.P + kSTile - 1) / kSTile;
   const int64_t grid = tiles < nsm ? tiles : nsm;

@@ -447,7 +447,7 @@ int launch_tc_t(const TcArgs &a, const CUtensorMap &tmap, cudaStream_t stream) {
   const TcLayout L = tc_layout<TILES>(a.H, a.R);
   if (L.total > max_optin) return RSC_ERR_UNSUPPORTED;
   auto kern = romp_tc_kernel<TILES, KK>;
-  e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, L.total);
+  e = rsc_allow_smem(kern, (size_t)L.total);
   if (e != cudaSuccess) return rsc_cuda_fail(e);
   const int64_t groups = (a.P + (int64_t)TILES * kTile - 1) / ((int64_t)TILES * kTile);
   const int64_t grid = groups < nsm ? groups : nsm;

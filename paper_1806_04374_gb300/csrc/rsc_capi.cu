@@ -684,6 +684,22 @@ cudaError_t rsc_scratch_alloc(void **p, size_t bytes, cudaStream_t st) {
   return cudaMallocFromPoolAsync(p, bytes, pool, st);
 }
 
+cudaError_t rsc_allow_smem(const void *kern, size_t bytes) {
+  // what every block may have without asking, less a margin for static memory
+  if (bytes <= 46 * 1024) return cudaSuccess;
+  int dev = 0, optin = 0;
+  cudaFuncAttributes at;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess)
+    e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+  if (e == cudaSuccess) e = cudaFuncGetAttributes(&at, kern);
+  if (e != cudaSuccess) return e;
+  const int most = optin - (int)at.sharedSizeBytes;
+  if (most < 0 || bytes > (size_t)most) return cudaErrorInvalidValue;
+  if (at.maxDynamicSharedSizeBytes >= most) return cudaSuccess;
+  return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+}
+
 cudaError_t rsc_scratch_free(void *p, cudaStream_t st) { return cudaFreeAsync(p, st); }
 
 void rsc_scratch_trim() {

@@ -302,6 +302,17 @@ int rsc_launch_f32(const RompArgs &a, cudaStream_t stream);
 // Records a CUDA error text for rsc_last_cuda_error and returns RSC_ERR_CUDA.
 int rsc_cuda_fail(cudaError_t e);
 
+// Lets the current device launch `kern` with `bytes` of dynamic shared memory.
+// The attribute belongs to the function and is common to all host threads, so
+// every call sets the same value, the most that a block may have beside the
+// kernel's own static shared memory: a thread that set the size of its own
+// launch could lower it between another thread's setting and launch.
+cudaError_t rsc_allow_smem(const void *kern, size_t bytes);
+template <class... A>
+cudaError_t rsc_allow_smem(void (*kern)(A...), size_t bytes) {
+  return rsc_allow_smem(reinterpret_cast<const void *>(kern), bytes);
+}
+
 // Per-call device scratch of the coders and the K-SVD update: stream-ordered
 // allocations from a memory pool per device that the library owns and that
 // keeps its memory between calls (rsc_capi.cu).  rsc_scratch_trim gives the
