@@ -139,9 +139,9 @@ int rsc_encode(const rsc_dict *dict, const float *x, int64_t P, int32_t K, int32
  * For every atom m, each patch whose code uses m at angle r0 contributes the
  * column S_{-r0}(x_p - D_aug b_p), b_p = the patch's code without that (m, r0)
  * entry; the new atom is the first left singular vector of those columns,
- * computed as the leading eigenvector of their covariance (FP32 products,
- * FP64 sums, FP64 power iteration from the old atom, to convergence or 5000
- * iterations).  All atoms are updated from the dictionary `dict` and the same
+ * computed as the leading eigenvector of their covariance (columns, products
+ * and sums beyond FP32: C is off by some 1e-15 of its norm; FP64 power
+ * iteration from the old atom, to convergence or 5000 iterations).  All atoms are updated from the dictionary `dict` and the same
  * codes.  Readings of the paper: a patch using m more than once contributes
  * its occurrence with the largest |weight| (ties: earliest); an atom used by
  * no patch is reset to the unit-normalised patch with the largest coding
@@ -157,6 +157,10 @@ int rsc_encode(const rsc_dict *dict, const float *x, int64_t P, int32_t K, int32
  *   n_used    : device int32 [M] or NULL: patches that used each atom.
  *   stream    : cudaStream_t.  Returns after launch; scratch comes from the
  *               library's scratch pool (see the top of this file).
+ * The covariances' kernel waits between its warps, each time for a limited
+ * while (rsc_dict_set_limits).  A wait that runs out records RSC_ERR_TIMEOUT,
+ * which rsc_dict_check(dict, stream) reports, and the atom it worked for comes
+ * out as not-a-numbers: check before the new atoms are used.
  */
 int rsc_ksvd_update(const rsc_dict *dict, const float *x, int64_t P, int32_t K,
                     const int32_t *atom, const int32_t *angle_idx, const double *coef,
@@ -175,7 +179,9 @@ int rsc_ksvd_update(const rsc_dict *dict, const float *x, int64_t P, int32_t K,
  *               patches and codes).
  *   C         : device double [M][n][n] output, n = J (2 kmax + 1): the sum
  *               over this rank's columns of y y^T in the packed coordinates
- *               (overwritten).
+ *               (overwritten).  After a wait that ran out (see
+ *               rsc_ksvd_update), not-a-numbers for the atom in question:
+ *               rsc_dict_check(dict, stream) before the sums are exchanged.
  *   count     : device int32 [M] output: this rank's columns per atom.
  *   top_err, top_idx, top_vec : device outputs, ntop entries: this rank's
  *               patches of largest coding error ||x - D_aug b||^2 (float),
@@ -419,12 +425,13 @@ int rsc_tuning_table_lookup(const char *path, int32_t n, int32_t M, int32_t R, i
 /*
  * rsc_dict_set_limits -- diagnostic limits on `dict`, for testing the error
  * paths (a property of this library; the paper has no counterpart).
- *   pipeline_wait_ns : limit of the waits between the FP16 scoring kernel's
- *            producer, MMA and epilogue warps; a wait that runs out records
+ *   pipeline_wait_ns : limit of the waits between the producer, MMA and
+ *            epilogue warps of the FP16 scoring kernel and of the K-SVD
+ *            covariance kernel; a wait that runs out records
  *            RSC_ERR_TIMEOUT (reported by rsc_dict_check), stops the kernel's
  *            loops and drains what it issued (those waits keep the default 2 s).
- *            The outputs of an rsc_encode that ran into it are undefined.
- *            0 = the default, 2 s.
+ *            The outputs of an rsc_encode that ran into it are undefined; an
+ *            atom's covariance is not-a-numbers.  0 = the default, 2 s.
  *   scratch_limit : largest per-call scratch (bytes) the FP16 path may take;
  *            a call that needs more returns RSC_ERR_OOM before any device
  *            work, as if the allocator had refused.  0 = no limit.

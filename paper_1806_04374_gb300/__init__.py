@@ -219,8 +219,9 @@ def rsc_dict_set_timing(handle: int, enable) -> int:
 
 
 def rsc_dict_set_limits(handle: int, pipeline_wait_ns: int = 0, scratch_limit: int = 0) -> int:
-    """Diagnostic limits for testing the error paths (0 = default): the FP16
-    scoring kernel's pipeline wait limit and the FP16 path's scratch budget."""
+    """Diagnostic limits for testing the error paths (0 = default): the wait
+    limit of the FP16 scoring and K-SVD covariance kernels' pipelines and the
+    FP16 path's scratch budget."""
     return load_library().rsc_dict_set_limits(ctypes.c_void_p(handle), int(pipeline_wait_ns),
                                               int(scratch_limit))
 

@@ -70,6 +70,7 @@ struct KsvdArgs {
   int *state;       // [split][M] what a slice's partial sum is (null: kCvFull64 all)
   int *expo;        // [split][M][128] exponents of a kCvPair slice's rows
   int *err;         // the dictionary's device error word
+  uint64_t wait_ns; // limit of the tensor-core kernel's pipeline waits
   float *new_coef;  // [M][H][J][2]
   int32_t *n_used;  // [M] or null
   // the patches of largest coding error (descending, ties: smaller index),
@@ -81,7 +82,7 @@ struct KsvdArgs {
   float *top_vec;   // [ntop][H][J][2]
 };
 
-enum : int { kCvPair = 0, kCvFull64 = 1, kCvNone = 2 };
+enum : int { kCvPair = 0, kCvFull64 = 1, kCvNone = 2, kCvFailed = 3 };
 
 constexpr int kTopMax = 64;  // patches kept for the resets (unused atoms beyond: unchanged)
 
@@ -443,7 +444,10 @@ __global__ void __launch_bounds__(kCovThreads) ksvd_cov_kernel(const KsvdArgs a)
 // 200,000 patches, K = 5, M = 128, n = 102, R = 64 (10^6 samples): 1.07 ms, and
 // the whole accumulation and update 1.63 ms (6.86 ms with every covariance on
 // the CUDA cores); C off by 1.8e-15 of its norm, 1.9e-15 there.
-// Every wait is bounded.
+// Every wait is bounded.  One that runs out is reported twice: in the
+// dictionary's error word, and as a slice without a sum (kCvFailed), which
+// makes all of its atom's C not a number, so that neither the covariance nor
+// what is added to it or made of it passes for a result.
 constexpr int kTcvBuild = 15, kTcvSum = 8;  // warps
 constexpr int kTcvThreads = 32 * (kTcvBuild + kTcvSum + 1);  // six warps a scheduler: 80 registers
 constexpr int kTcvSamples = 64;          // samples of a stage
@@ -455,7 +459,7 @@ constexpr int kTcvMaxN = 112;            // packed lengths up to here
 constexpr int kTcvUnits = 5;             // pieces of eight columns of a summing warp
 constexpr int kTcvTwMax = 28 * 1024;     // steering factors kept in shared memory (bytes)
 constexpr int kTcvPlaces = kTcvSum * 8 * kTcvUnits * 32;  // of a slice's sums
-constexpr uint64_t kTcvWaitNs = 2000000000ull;
+constexpr uint64_t kTcvWaitNs = 2000000000ull;  // drain waits (and the default pipeline limit)
 enum : int { kCvFull = 0, kCvEmpty = 2, kCvXFull = 4, kCvXFree = 5, kCvAccFull = 6, kCvAccFree = 7, kCvRec = 8, kCvBars = 12 };
 constexpr int kTcvBarOff = 2 * kTcvStage;
 constexpr int kTcvScOff = kTcvBarOff + 128;       // [128] exponents of the rows
@@ -620,6 +624,7 @@ __global__ void __launch_bounds__(kTcvThreads, 1) ksvd_cov_tc_kernel(const KsvdA
   const int nst = (ns + kTcvSamples - 1) / kTcvSamples;
   auto fail = [&]() {
     *s_abort = 1;
+    a.state[slice] = kCvFailed;
     if (a.err) atomicCAS(a.err, 0, RSC_ERR_TIMEOUT);
   };
 
@@ -649,8 +654,8 @@ __global__ void __launch_bounds__(kTcvThreads, 1) ksvd_cov_tc_kernel(const KsvdA
                           tc::desc_at(d0, j * kTcvSlice + ks * 32), idesc,
                           clear && ks == 0 ? 0u : 1u);
         };
-        if (*s_abort || !tc::mbar_wait_bounded(bar(kCvFull + b), (st >> 1) & 1, kTcvWaitNs) ||
-            (st > 0 && !tc::mbar_wait_bounded(bar(kCvXFree), 1, kTcvWaitNs))) {
+        if (*s_abort || !tc::mbar_wait_bounded(bar(kCvFull + b), (st >> 1) & 1, a.wait_ns) ||
+            (st > 0 && !tc::mbar_wait_bounded(bar(kCvXFree), 1, a.wait_ns))) {
           fail();
           break;
         }
@@ -660,12 +665,12 @@ __global__ void __launch_bounds__(kTcvThreads, 1) ksvd_cov_tc_kernel(const KsvdA
         for (int q = 0; q < kRest; ++q) product(3, rest[q][0], rest[q][1], q == 0);
         tc::mma_commit(bar(kCvXFull));
         bool ok = !(opens && win > 0) ||
-                  tc::mbar_wait_bounded(bar(kCvAccFree), (win - 1) & 1, kTcvWaitNs);
+                  tc::mbar_wait_bounded(bar(kCvAccFree), (win - 1) & 1, a.wait_ns);
         tc::fence_after_sync();
         if (ok) {
 #pragma unroll
           for (int q = 0; q < 3; ++q) product(low[q][0], low[q][1], low[q][2], opens && q < 2);
-          ok = tc::mbar_wait_bounded(bar(kCvXFree), 0, kTcvWaitNs);
+          ok = tc::mbar_wait_bounded(bar(kCvXFree), 0, a.wait_ns);
         }
         tc::fence_after_sync();
         if (ok) {
@@ -707,7 +712,7 @@ __global__ void __launch_bounds__(kTcvThreads, 1) ksvd_cov_tc_kernel(const KsvdA
     for (int u = 0; u < 8 * kTcvUnits; ++u) third[u] = 0.0f;
     bool ok = true;
     auto wait = [&](int i, int parity) {
-      const bool done = !*s_abort && tc::mbar_wait_bounded(bar(i), parity, kTcvWaitNs);
+      const bool done = !*s_abort && tc::mbar_wait_bounded(bar(i), parity, a.wait_ns);
       ok = __all_sync(0xffffffffu, done);
       tc::fence_after_sync();
       return ok;
@@ -808,11 +813,11 @@ __global__ void __launch_bounds__(kTcvThreads, 1) ksvd_cov_tc_kernel(const KsvdA
     for (int st = 0; st < nst; ++st) {
       const int b = st & 1;
       bool done = !*s_abort && (st < 2 || tc::mbar_wait_bounded(bar(kCvEmpty + b),
-                                                                ((st >> 1) - 1) & 1, kTcvWaitNs));
+                                                                ((st >> 1) - 1) & 1, a.wait_ns));
       if (__all_sync(0xffffffffu, done)) {
         fetch(st + 2);
         fetched = min(nst, st + 3);
-        done = tc::mbar_wait_bounded(bar(kCvRec + (st & 3)), (st >> 2) & 1, kTcvWaitNs);
+        done = tc::mbar_wait_bounded(bar(kCvRec + (st & 3)), (st >> 2) & 1, a.wait_ns);
       }
       if (!__all_sync(0xffffffffu, done)) {
         if (lane == 0) fail();
@@ -936,6 +941,8 @@ __global__ void ksvd_cov_pair_sum_kernel(const KsvdArgs a, int N) {
         lo = __fadd_rn(lo, __fadd_rn(f * r, __fadd_rn(s1.lo, s2.lo)));
       } else if (state == kCvFull64) {
         other += from[(size_t)i * n + j];
+      } else if (state == kCvFailed) {
+        other = __longlong_as_double(0x7ff8000000000000ll);
       }
     }
     const double s = ((double)hi + (double)mid) + ((double)lo + other);
@@ -1152,6 +1159,7 @@ int ksvd_setup(const rsc_dict *dict, int64_t P, int K, KsvdArgs &a) {
   a.n = dict->J + 2 * dict->kmax * dict->J;
   if (a.n > kMaxPacked || a.M > kMaxAtomsKsvd) return RSC_ERR_UNSUPPORTED;
   a.err = dict->err;
+  a.wait_ns = dict->wait_ns ? dict->wait_ns : kTcvWaitNs;
   a.d = dict->d;
   a.tw = dict->tw;
   return RSC_OK;

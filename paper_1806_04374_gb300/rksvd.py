@@ -14,7 +14,25 @@ import os
 
 import numpy as np
 
-from . import KSVD_TOP, Dictionary, encode, ksvd_accumulate, ksvd_finish, ksvd_update
+from . import (KSVD_TOP, Dictionary, RscError, encode, ksvd_accumulate, ksvd_finish, ksvd_update,
+               rsc_dict_check)
+
+
+def device_status(dic: Dictionary) -> int:
+    """Waits for the current stream and returns the first error that the
+    device recorded on `dic` since the last check (rsc_dict_check; 0: none)."""
+    import torch
+    return rsc_dict_check(dic.handle, int(torch.cuda.current_stream().cuda_stream))
+
+
+def _agree(status: int, group, device) -> int:
+    """The worst status (0 or a negative code) of the ranks of `group`."""
+    import torch
+    import torch.distributed as dist
+    t = torch.tensor([status], dtype=torch.int64,
+                     device=device if dist.get_backend(group) == "nccl" else "cpu")
+    dist.all_reduce(t, op=dist.ReduceOp.MIN, group=group)
+    return int(t.item())
 
 
 def merge_top(errs, gidxs, vecs, ntop: int = KSVD_TOP):
@@ -52,9 +70,15 @@ def update_distributed(dic: Dictionary, x, codes: dict, group=None, offset: int 
     """One R-K-SVD update with this rank's patches x (global indices start at
     `offset`) and codes: accumulate here, sum the covariances and counts over
     `group`, merge the largest-error lists, finish.  With group None it is
-    the single-GPU update.  Returns (new atoms, n_used)."""
+    the single-GPU update.  A device-side error on any rank raises RscError on
+    every rank before anything is summed.  Returns (new atoms, n_used)."""
     import torch
     acc = ksvd_accumulate(dic, x, codes)
+    status = device_status(dic)
+    if group is not None:
+        status = _agree(status, group, x.device)
+    if status != 0:
+        raise RscError(status, "rsc_ksvd_accumulate")
     if group is None:
         return ksvd_finish(dic, acc["C"], acc["count"], acc["top_idx"], acc["top_vec"])
     _all_reduce_sum(acc["C"], group)
@@ -115,7 +139,10 @@ def learn(x, d0, R: int, K: int, iters: int, precision: str = "f16", callback=No
     file).  The loop draws no random numbers and its kernels give the same
     result on every run, so that is its whole state: with resume=True and an
     existing file, learning continues after the saved iteration and ends
-    with the atoms of an uninterrupted run, bit for bit."""
+    with the atoms of an uninterrupted run, bit for bit.
+
+    A device-side error (a bounded wait of a kernel that ran out) raises
+    RscError before the atoms it touched are used or saved."""
     import torch
     d = d0.contiguous()
     n = d.shape[2] * (2 * (d.shape[1] - 1) + 1)
@@ -133,7 +160,10 @@ def learn(x, d0, R: int, K: int, iters: int, precision: str = "f16", callback=No
             new, used = ksvd_update(dic, x, codes)
         else:
             new, used = update_distributed(dic, x, codes, group, offset)
-        torch.cuda.current_stream().synchronize()
+        # (also waits for the update)
+        status = device_status(dic)
+        if status != 0:
+            raise RscError(status, "R-K-SVD iteration")
         rec = {"iter": it, "mse": float(codes["resid_norm2"].double().mean().item()) / n,
                "unused": int((used == 0).sum().item())}
         history.append(rec)
@@ -145,7 +175,9 @@ def learn(x, d0, R: int, K: int, iters: int, precision: str = "f16", callback=No
             save_checkpoint(checkpoint, d.cpu().numpy(), it + 1, history, R, K)
     dic = Dictionary(d, R)
     codes = encode(dic, x, K, precision)
-    torch.cuda.current_stream().synchronize()
+    status = device_status(dic)
+    if status != 0:
+        raise RscError(status, "rsc_encode")
     history.append({"iter": iters, "mse": float(codes["resid_norm2"].double().mean().item()) / n,
                     "unused": None})
     dic.close()
