@@ -187,6 +187,23 @@ __device__ __forceinline__ unsigned char *smem_align16(unsigned char *p) {
   return reinterpret_cast<unsigned char *>((reinterpret_cast<uintptr_t>(p) + 15) & ~uintptr_t(15));
 }
 
+// ||e||^2 of the residual at E (each lane its own entries, as it wrote them) in
+// FP64, rounded once: infinity past FP32's range.
+__device__ __noinline__ float coding_error64(const float4 *E, int HJ, int lane) {
+  double s = 0.0;
+  bool some = false;
+  for (int e = lane; e < HJ; e += 32) some |= E[e].x != 0.0f || E[e].y != 0.0f;
+  if (!__any_sync(0xffffffffu, some)) return 0.0f;  // (NaN is not 0)
+  for (int e = lane; e < HJ; e += 32) {
+    const float4 v = E[e];
+    const double re = (double)v.x + (double)v.z, im = (double)v.y + (double)v.w;
+    s = fma(re, re, fma(im, im, s));
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+  return (float)s;
+}
+
 template <bool TW>
 __global__ void __launch_bounds__(kFillThreads) ksvd_fill_kernel(const KsvdArgs a) {
   // [kFillChunk][K] code (weight hi, lo, atom or -1, angle); [M] next slot of
@@ -269,7 +286,10 @@ __global__ void __launch_bounds__(kFillThreads) ksvd_fill_kernel(const KsvdArgs 
       n2 = df_add(n2, df_add(df_mul(re, re), df_mul(im, im)));
     }
     n2 = df_warp_sum(n2);
-    if (lane == 0) a.err2[p] = n2.hi;
+    // squares outside FP32's range (infinite, or tails lost below it): FP64
+    float err = n2.hi;
+    if (!(err > 1e-30f && err < 1e38f)) err = coding_error64(a.E + p * HJ, HJ, lane);
+    if (lane == 0) a.err2[p] = err;
   }
   __syncthreads();
   for (int i = threadIdx.x; i < np * K; i += kFillThreads) {
