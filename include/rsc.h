@@ -293,7 +293,8 @@ int rsc_classify_images(const rsc_dict *const *dicts, int32_t C, const rsc_basis
 /*
  * rsc_reconstruct -- the coded patches back in steerable coordinates:
  * x_hat_p = sum_i a_i S_{r_i} d_{m_i} (Sec. II-C's sparse code with the
- * steering of Eq. (Sr)), accumulated in double-float.
+ * steering of Eq. (Sr)); every entry is rounded once to float32 from a sum
+ * kept in FP64 or to 2^-27 of the entry.
  *   atom, angle_idx, coef : device, P x K, as rsc_encode writes them (steps
  *            with atom = -1 are skipped); int32 / int32 / double.
  *   out    : device, P x (kmax+1) x J x 2 floats (half spectra; the Im of

@@ -4,8 +4,8 @@
 //
 // rsc_reconstruct: x_hat_p = sum_i a_i S_{r_i} d_{m_i} for each patch's code
 //   (steering of Eq. (Sr): harmonic k of an atom times exp(-i k 2 pi r / R)),
-//   accumulated to about 48 bits from the dictionary's FP32 atoms and its
-//   double-float steering factors, rounded once to FP32.
+//   from the dictionary's FP32 atoms and its double-float steering factors;
+//   every entry its FP64 value rounded to FP32 (to 2^-24 + 2^-27 of itself).
 // rsc_synthesize: pixels = Phi x_hat over the circular patch, a tiled FP32
 //   matrix product with the basis's real synthesis matrix (rows in the half
 //   spectrum's order, the packing weights folded in).
@@ -42,18 +42,19 @@ __device__ __forceinline__ float2 halves(f32x2 v) {
 
 // ------------------------------------------------------------ reconstruct
 //
-// Bound by FP32 issue: 20 operations per term and entry, two to an
+// Bound by FP32 issue: 32 operations per term and entry, two to an
 // instruction.  A warp takes a tile of patches, a lane up to kRecEntries
 // entries of one patch's harmonic: it forms the steered weights
 // a_i e^{-i k theta_i} in double-float once per term and applies them to its
-// entries' FP32 atoms, accumulating to about 48 bits.
-// 10^6 patches of 54 entries, K = 5: 0.41 ms (the operations themselves 0.13
+// entries' FP32 atoms, accumulating to about 60 bits.
+// 10^6 patches of 54 entries, K = 5: 0.53 ms (the operations themselves 0.21
 // at the FP32 peak; a two-element FMA takes 2.3 cycles, so it saves issue
 // slots and no time on the pipe), against 7.0 ms for FP64 throughout (15
 // operations per term on a pipe of 1/64 of the FP32 rate, every factor formed
-// again for every entry); the memory floor is 75 us.  A lane per two entries
-// with the steered weights kept in shared memory took 0.52 ms, with one block
-// per tile and barriers between the phases 0.60.
+// again for every entry); the memory floor is 75 us.  With two floats for an
+// accumulator (48 bits, 0.42 ms) entries that cancel to 2^-20 of the weights
+// came out up to 7 x 2^-24 off.  Four entries a lane 0.73 ms, a third block an
+// SM (80 registers, spills) 0.55; of the time 5% are the entries in FP64.
 constexpr int kRecThreads = 256;
 constexpr int kRecTile = 32;   // patches per warp and tile
 constexpr int kRecEntries = 6;
@@ -61,19 +62,25 @@ constexpr int kRecEntries = 6;
 // Accumulators of products w d, |sum| < 2^(E-1) throughout: acc starts at
 // 1.5 2^E, so that every partial sum stays in [2^E, 2^(E+1)) and acc holds it
 // rounded to a multiple of 2^(E-23), exactly tracked: acc - t and the
-// remainder w.hi d - (t - acc) (one FMA) are exact, and c collects the
-// remainders and the lo part.  Five operations instead of the eleven of
-// TwoProd + TwoSum; the error is a few 2^(E-48).
-__device__ __forceinline__ void acc_prod2(f32x2 &acc, f32x2 &c, f32x2 whi, f32x2 wlo, f32x2 d) {
+// remainder l = w.hi d - (t - acc) (one FMA) are exact.  The remainders, up to
+// 2K of 2^(E-24), are summed the same way from 1.5 2^(E-17), and r collects what
+// that leaves and the lo parts: eight operations instead of the eleven of
+// TwoProd + TwoSum.  The weights are off by 2^-46 of themselves and r, below
+// 2^(E-25), is rounded 4K times: (K + 1) 2^(E-48) in all.
+__device__ __forceinline__ void acc_prod2(f32x2 &acc, f32x2 &c, f32x2 &r, f32x2 whi, f32x2 wlo,
+                                          f32x2 d) {
+  const f32x2 minus1 = pack2(-1.0f, -1.0f);
   const f32x2 t = fma2(whi, d, acc);
-  const f32x2 l = fma2(whi, d, fma2(t, pack2(-1.0f, -1.0f), acc));
+  const f32x2 l = fma2(whi, d, fma2(t, minus1, acc));
   acc = t;
-  c = fma2(wlo, d, add2(c, l));
+  const f32x2 u = add2(c, l);
+  r = fma2(wlo, d, add2(r, add2(l, fma2(u, minus1, c))));
+  c = u;
 }
 
 // One entry in FP64 straight from the code, for patches and entries outside
 // the range of acc_prod2 (weights that are not finite or far from 1; an entry
-// that cancels to less than 2^-22 of its terms).
+// that cancels so far that the accumulators' error would show).
 __device__ __forceinline__ float2 reconstruct_entry(const float *__restrict__ d,
                                                  const float *__restrict__ tw, int H, int HJ, int R,
                                                  int K, const int32_t *__restrict__ atom,
@@ -101,7 +108,7 @@ __device__ __forceinline__ float2 reconstruct_entry(const float *__restrict__ d,
 // aligned output).  A harmonic's J entries are split over nsub lanes, `per`
 // each (the last fewer; even with PAIRS).
 template <bool PAIRS>
-__global__ void __launch_bounds__(kRecThreads)
+__global__ void __launch_bounds__(kRecThreads, 2)
     reconstruct_kernel(const float *__restrict__ d, const float *__restrict__ tw, int H, int J,
                        int R, int64_t P, int K, int tile, int nsub, int per,
                        const int32_t *__restrict__ atom, const int32_t *__restrict__ angle_idx,
@@ -131,7 +138,7 @@ __global__ void __launch_bounds__(kRecThreads)
                          m < 0 ? 0 : m * HJ);
     }
     __syncwarp();
-    // lane l: 1.5 2^E of patch l (0: FP64)
+    // lane l: 1.5 2^E of patch l (0: FP64; negative: nothing coded, zeros)
     float sigl = 0.0f;
     if (lane < np) {
       float sum = 0.0f;
@@ -140,6 +147,7 @@ __global__ void __launch_bounds__(kRecThreads)
       int E = 0;
       (void)frexpf(1.01f * sum, &E);
       if (sum > 1e-20f && sum < 1e25f) sigl = 1.5f * exp2f((float)(E + 1));  // NaN: 0
+      if (sum == 0.0f) sigl = -1.5f;
     }
     for (int base = 0; base < np * items; base += 32) {
       const int it = base + lane;
@@ -148,13 +156,15 @@ __global__ void __launch_bounds__(kRecThreads)
       if (it >= np * items) continue;
       const int k = ks / nsub, e0 = k * J + (ks - k * nsub) * per;
       const int cnt = min(per, (k + 1) * J - e0);
-      f32x2 acc[kRecEntries], cor[kRecEntries];
+      f32x2 acc[kRecEntries], cor[kRecEntries], rem[kRecEntries];
+      const float sig2 = sig * 7.62939453125e-6f;  // 1.5 2^(E-17)
 #pragma unroll
       for (int j = 0; j < kRecEntries; ++j) {
         acc[j] = pack2(sig, sig);
-        cor[j] = 0;
+        cor[j] = pack2(sig2, sig2);
+        rem[j] = 0;
       }
-      if (sig != 0.0f) {
+      if (sig > 0.0f) {
         const float2 *dp = reinterpret_cast<const float2 *>(d) + e0;
         const int4 *ap = s_a + pl * K;
 #pragma unroll 1
@@ -182,32 +192,39 @@ __global__ void __launch_bounds__(kRecThreads)
           for (int j = 0; j < kRecEntries; ++j) {
             // (re, im) += a c (dr, di) + (a s, -a s) (di, dr); k = 0 holds
             // real numbers: the table's sine and the atoms' di are 0 there
-            acc_prod2(acc[j], cor[j], ch, cl, pack2(dv[j].x, dv[j].y));
-            acc_prod2(acc[j], cor[j], sh, sl, pack2(dv[j].y, dv[j].x));
+            acc_prod2(acc[j], cor[j], rem[j], ch, cl, pack2(dv[j].x, dv[j].y));
+            acc_prod2(acc[j], cor[j], rem[j], sh, sl, pack2(dv[j].y, dv[j].x));
           }
         }
       }
-      // sig = 1.5 2^E: below 2^-22 2^E the accumulator's error would show
-      const float tiny = sig * 1.589457194e-7f;  // 2^-22 / 1.5
+      // sig = 1.5 2^E: entries below (K + 1) 2^(E-21) would show more than 2^-27
+      // of themselves of the accumulators' error, beside the one rounding to
+      // FP32, and are formed in FP64 (the line lies at 6 to 12 x 10^-6 sum |a_i|
+      // for K = 5: about 0.01% of the values of random atoms are below it)
+      const float tiny = sig * ((float)(K + 1) * 3.178914388e-7f);  // (K + 1) 2^-21 / 1.5
       float2 o[kRecEntries];
-      bool low = sig == 0.0f;
+      unsigned low = 0;
 #pragma unroll
       for (int j = 0; j < kRecEntries; ++j) {
-        const float2 h = halves(add2(acc[j], pack2(-sig, -sig))), c = halves(cor[j]);
-        o[j] = make_float2(__fadd_rn(h.x, c.x), __fadd_rn(h.y, c.y));
+        const float2 h = halves(add2(acc[j], pack2(-sig, -sig)));
+        const float2 c = halves(add2(cor[j], pack2(-sig2, -sig2))), q = halves(rem[j]);
+        const df x = two_sum(h.x, c.x), y = two_sum(h.y, c.y);
+        o[j] = make_float2(__fadd_rn(x.hi, __fadd_rn(x.lo, q.x)),
+                           __fadd_rn(y.hi, __fadd_rn(y.lo, q.y)));
         // (an exact zero is what it is)
-        low |= (fabsf(o[j].x) < tiny && (o[j].x != 0.0f || c.x != 0.0f)) ||
-               (fabsf(o[j].y) < tiny && (o[j].y != 0.0f || c.y != 0.0f));
+        const bool lx = fabsf(o[j].x) < tiny && (x.hi != 0.0f || q.x != 0.0f);
+        const bool ly = fabsf(o[j].y) < tiny && (y.hi != 0.0f || q.y != 0.0f);
+        if (lx || ly || sig == 0.0f) low |= 1u << j;
       }
-      if (low) {
-#pragma unroll 1
-        for (int j = 0; j < cnt; ++j) {
-          const float2 q = reconstruct_entry(d, tw, H, HJ, R, K, atom, angle_idx, coef, p0 + pl,
-                                             e0 + j, k);
+      low &= (1u << cnt) - 1u;
+      while (low) {
+        const int j = __ffs(low) - 1;
+        low &= low - 1;
+        const float2 q = reconstruct_entry(d, tw, H, HJ, R, K, atom, angle_idx, coef, p0 + pl,
+                                           e0 + j, k);
 #pragma unroll
-          for (int u = 0; u < kRecEntries; ++u)
-            if (u == j) o[u] = q;
-        }
+        for (int u = 0; u < kRecEntries; ++u)
+          if (u == j) o[u] = q;
       }
       float2 *op = reinterpret_cast<float2 *>(out) + (p0 + pl) * HJ + e0;
 #pragma unroll
