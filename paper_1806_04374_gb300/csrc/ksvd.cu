@@ -445,11 +445,12 @@ __global__ void __launch_bounds__(kCovThreads) ksvd_cov_kernel(const KsvdArgs a)
 // values y = b0 + ... + b5: b0, b1, b2 and b3 multiples of 2^-8, 2^-16, 2^-24
 // and 2^-32 below 2^-1, 2^-9, 2^-17 and 2^-24, b4 and b5 what is left, 8 bits
 // each.  The 26 products b_i b_j^T down to 2^-53 are summed by order i + j:
-// orders 0 to 3 are integers (in units of 2^-16, 2^-24, 2^-32, 2^-40) whose sums
-// stay below 2^24 for a window of samples, so the FP32 accumulator holds them
-// exactly; the rest, 2^-32 of the whole, is summed as it comes.  Orders 0 to 2
-// have an accumulator each; order 3 and the rest take turns in a fourth, read
-// out after each turn.  A slice's sums are kept in three floats without loss
+// orders 0 to 3 are integers (in units of 2^-16, 2^-24, 2^-32, 2^-40), at most
+// 2^14, 2^15, 3 2^14 and 5 2^14 a sample.  Sums of orders 0 to 2 stay below 2^24
+// for a window of samples, those of order 3 for three stages of it, so FP32
+// holds them exactly; the rest, 2^-32 of the whole, is summed as it comes.
+// Orders 0 to 2 have an accumulator each; order 3 and the rest take turns in a
+// fourth, read out after each turn.  A slice's sums are kept in three floats without loss
 // but for the third's own rounding, 2^-24 of 2^-28 (FP64 at 64 cycles an
 // instruction held the accumulators up).
 //
@@ -474,7 +475,11 @@ constexpr int kTcvSamples = 64;          // samples of a stage
 constexpr int kTcvSlices = 6;
 constexpr int kTcvSlice = 128 * 128;     // one slice of a stage (bytes)
 constexpr int kTcvStage = kTcvSlices * kTcvSlice;
-constexpr int kTcvStages = 5;            // stages per window: 3 * 2^14 * 320 < 2^24
+constexpr int kTcvStages = 5;            // stages per window: order 2, 3 * 2^14 * 320 < 2^24
+constexpr int kTcvThird = 3;             // of these, order 3 at once: 5 * 2^14 * 192 < 2^24
+// the sum of order 3 that two stages more leave below 2^24 (units of 2^-40)
+constexpr float kTcvThirdMax =
+    (float)((1 << 24) - 5 * (1 << 14) * kTcvSamples * (kTcvStages - kTcvThird)) / 1099511627776.0f;
 constexpr int kTcvMaxN = 112;            // packed lengths up to here
 constexpr int kTcvUnits = 5;             // pieces of eight columns of a summing warp
 constexpr int kTcvTwMax = 28 * 1024;     // steering factors kept in shared memory (bytes)
@@ -722,7 +727,8 @@ __global__ void __launch_bounds__(kTcvThreads, 1) ksvd_cov_tc_kernel(const KsvdA
     // Sums of this lane's row, in three parts in their places of Cpart: two
     // that take the orders 0 to 3 exactly and one for the rest and what the
     // other two lose.  (Atomic adds so that nothing waits for them: a place
-    // has one thread.)  Order 3 is summed in registers over a window, exactly.
+    // has one thread.)  Order 3 is summed in registers over a window, exactly:
+    // in two parts where one could pass 2^24.
     float2 *sum = reinterpret_cast<float2 *>(a.Cpart + slice * a.stride) +
                   (size_t)sw * 8 * kTcvUnits * 32 + lane;
     float *rest = reinterpret_cast<float *>(a.Cpart + slice * a.stride) + 2 * kTcvPlaces +
@@ -730,7 +736,7 @@ __global__ void __launch_bounds__(kTcvThreads, 1) ksvd_cov_tc_kernel(const KsvdA
     float third[8 * kTcvUnits];
 #pragma unroll
     for (int u = 0; u < 8 * kTcvUnits; ++u) third[u] = 0.0f;
-    bool ok = true;
+    bool ok = true, moved = false;
     auto wait = [&](int i, int parity) {
       const bool done = !*s_abort && tc::mbar_wait_bounded(bar(i), parity, a.wait_ns);
       ok = __all_sync(0xffffffffu, done);
@@ -744,6 +750,30 @@ __global__ void __launch_bounds__(kTcvThreads, 1) ksvd_cov_tc_kernel(const KsvdA
     };
     for (int st = 0; st < nst && ok; ++st) {
       const int win = st / kTcvStages;
+      // sums of order 3 that the window's other stages could take past 2^24
+      // move to their places first (equal columns; others stay far below)
+      if (st - win * kTcvStages == kTcvThird) {
+        float most = 0.0f;
+#pragma unroll
+        for (int u = 0; u < 8 * kTcvUnits; ++u) most = fmaxf(most, fabsf(third[u]));
+        moved = __any_sync(0xffffffffu, most > kTcvThirdMax);
+        if (moved) {
+#pragma unroll
+          for (int s = 0; s < kTcvUnits; ++s) {
+            if (column(s) < N) {
+#pragma unroll
+              for (int u = 0; u < 8; ++u) {
+                float2 *to = &sum[(8 * s + u) * 32];
+                const float2 old = win ? *to : make_float2(0.0f, 0.0f);
+                const df t = two_sum(old.y, third[8 * s + u]);
+                *to = make_float2(old.x, t.hi);
+                if (win) atomicAdd(&rest[(8 * s + u) * 32], t.lo);  // (else 0)
+                third[8 * s + u] = 0.0f;
+              }
+            }
+          }
+        }
+      }
       for (int turn = 0; turn < 2; ++turn) {
         if (!wait(kCvXFull, turn)) break;
 #pragma unroll
@@ -786,7 +816,7 @@ __global__ void __launch_bounds__(kTcvThreads, 1) ksvd_cov_tc_kernel(const KsvdA
             float2 old[8];
 #pragma unroll
             for (int u = 0; u < 8; ++u)
-              old[u] = win ? sum[(8 * s + u) * 32] : make_float2(0.0f, 0.0f);
+              old[u] = win || moved ? sum[(8 * s + u) * 32] : make_float2(0.0f, 0.0f);
             uint32_t v2[8];
             tmem_ld8(tlane + 2 * N + c0, v2);
             tc::tmem_wait_ld();
