@@ -37,3 +37,25 @@ def test_odd_angles(rsc, case):
     x, _ = synth.make_patches(d, P, min(4, K), 0.1, 8100 + P)
     g = run_gpu(rsc, x, d, R, K, precision)
     check(x, d, R, K, g, TOL)
+
+
+@pytest.mark.parametrize("R", [31, 33, 64, 128])
+def test_codes_do_not_depend_on_the_patches_before(rsc, R):
+    """A warp chooses the pass over the scores by its last step: patches near
+    pairs of equal atoms and others, in turn, in reverse and apart, are coded
+    the same, bit for bit."""
+    import torch
+    d = synth.make_dictionary(24, 6, 8, 7300)
+    d = np.concatenate([d, d[:8]])
+    P = 8000
+    near, _ = synth.make_patches(d[:8], P, 2, 0.05, 7301)
+    far, _ = synth.make_patches(d[8:24], P, 2, 0.05, 7302)
+    x = torch.from_numpy(np.where((np.arange(P) % 7 < 3)[:, None, None, None], near, far)).cuda()
+    dic = rsc.Dictionary(torch.from_numpy(d).cuda(), R)
+    got = rsc.encode(dic, x, 3, "fp32")
+    back = rsc.encode(dic, x.flip(0).contiguous(), 3, "fp32")
+    part = rsc.encode(dic, x[:500].contiguous(), 3, "fp32")
+    for k in got:
+        assert torch.equal(got[k], back[k].flip(0)), k
+        assert torch.equal(got[k][:500], part[k]), k
+    dic.close()
