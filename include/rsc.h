@@ -120,7 +120,8 @@ int rsc_dict_dims(const rsc_dict *dict, rsc_dims *dims);
  *   prec      : RSC_FP32, RSC_FP32_PRUNE or RSC_F16_RESCORE.  RSC_F16_RESCORE takes packed
  *               lengths J (2 kmax + 1) <= 256 and K <= 8 (RSC_ERR_UNSUPPORTED
  *               otherwise); the dictionary's tables for it are built by
- *               rsc_dict_create when the sizes allow.
+ *               rsc_dict_create when the sizes allow (RSC_ERR_OOM when device
+ *               memory for them was refused then).
  *   atom      : device int32 [P x K], atom index m per step, -1 if none.
  *   angle_idx : device int32 [P x K], angle index r in [0, R), -1 if none.
  *   angle     : device float [P x K] or NULL, the angle 2*pi*r/R in radians.

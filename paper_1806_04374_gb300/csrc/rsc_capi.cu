@@ -14,6 +14,7 @@
 #include <vector>
 
 #include "df.cuh"
+#include "dict_tables.h"
 #include "rsc_internal.h"
 #include "rsc_trace.h"
 
@@ -339,17 +340,17 @@ int build_tc_tables(rsc_dict *d, cudaStream_t st) {
   d->Rr = R % 2 == 0 ? R / 2 : R;
   const int64_t nrow = (int64_t)d->Rr * M * L, ng = (int64_t)M * M * R;
   // the refine's tables share one allocation, at d->xgram
-  auto al = [](size_t v) { return (v + 255) & ~(size_t)255; };
-  const size_t bx = al((size_t)M * M * H * sizeof(float4)), ba = al((size_t)M * sizeof(float2)),
-               br = al((size_t)nrow * 2 * sizeof(float)), bg = (size_t)ng * sizeof(float2);
-  const bool gram = bg <= kGramMax;
-  unsigned char *tables = nullptr;
-  if (e == cudaSuccess) e = cudaMalloc(&tables, bx + ba + br + (gram ? bg : 0));
+  RefineTables t = plan_refine_tables(M, H, R, d->Rr, L);
+  void *base = nullptr;
+  if (e == cudaSuccess)
+    e = alloc_refine_tables(t, [](void **p, size_t bytes) { return cudaMalloc(p, bytes); }, &base);
   if (e == cudaSuccess) {
+    cudaGetLastError();  // of a part that was refused
+    unsigned char *tables = static_cast<unsigned char *>(base);
     d->xgram = reinterpret_cast<float4 *>(tables);
-    d->anorm = reinterpret_cast<float2 *>(tables + bx);
-    d->rows = reinterpret_cast<float *>(tables + bx + ba);
-    d->gram = gram ? reinterpret_cast<float2 *>(tables + bx + ba + br) : nullptr;
+    d->anorm = reinterpret_cast<float2 *>(tables + t.xgram);
+    if (t.rows) d->rows = reinterpret_cast<float *>(tables + t.xgram + t.anorm);
+    if (t.gram) d->gram = reinterpret_cast<float2 *>(tables + t.xgram + t.anorm + t.rows);
   }
   if (e == cudaErrorMemoryAllocation) {
     cudaGetLastError();
@@ -367,8 +368,9 @@ int build_tc_tables(rsc_dict *d, cudaStream_t st) {
   const int64_t nx = (int64_t)M * M * H;
   xgram_kernel<<<(unsigned)((nx + T - 1) / T), T, 0, st>>>(d->d, M, J, H, d->xgram);
   anorm_kernel<<<(M + T - 1) / T, T, 0, st>>>(d->d, M, J, H, d->anorm);
-  refine_rows_kernel<<<(unsigned)((nrow + T - 1) / T), T, 0, st>>>(d->d, d->tw, M, J, d->kmax, R,
-                                                                   d->Rr, L, paired, d->rows);
+  if (d->rows)
+    refine_rows_kernel<<<(unsigned)((nrow + T - 1) / T), T, 0, st>>>(d->d, d->tw, M, J, d->kmax, R,
+                                                                     d->Rr, L, paired, d->rows);
   if (d->gram)
     gram_kernel<<<(unsigned)((ng + T - 1) / T), T, 0, st>>>(d->xgram, d->tw, M, H, R, d->gram);
   e = cudaGetLastError();
@@ -926,6 +928,7 @@ int encode_impl(const rsc_dict *dict, const RompArgs &a, int32_t prec, cudaStrea
   // FP16 tensor-core path, split per greedy step into a scoring kernel and a
   // per-patch refine kernel; patches it hands back are coded by the FP32 path
   if (!dict->steered_f16 || K > kTcMaxK || P >= ((int64_t)1 << 31)) return RSC_ERR_UNSUPPORTED;
+  if (!dict->rows) return RSC_ERR_OOM;  // refused when the dictionary was made
   // Independent groups of patches on their own streams: the scoring pass of
   // one group (tensor and ALU pipes, one CTA per SM) runs beside the refine
   // pass of another (latency-bound), so each hides part of the other.

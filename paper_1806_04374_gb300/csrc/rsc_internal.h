@@ -39,10 +39,10 @@ struct rsc_dict {
   // steered atoms as the refine reads them (romp_refine.cu): rows r*M + m of
   // row_len FP32 entries, hi plane then lo plane (double-float), without the
   // packing weights; r < Rr = R/2 for even R (half a turn changes the sign
-  // of the odd harmonics), else R
+  // of the odd harmonics), else R; null when the allocator refused them
   float *rows;
   int Rr;
-  float2 *gram;          // [M][M][R] double-float <S_r d_a, d_b>; null when over kGramMax bytes
+  float2 *gram;          // [M][M][R] double-float <S_r d_a, d_b>; null when over kGramMax bytes or refused
   int n;                 // packed real length J (2 kmax + 1)
   // per-phase timing (diagnostic): event pairs recorded around launches
   int timing;
@@ -73,7 +73,6 @@ constexpr int kTcKstLong = 256;  // row length for packed lengths 113..256 (plai
 constexpr int kTcOdd = 64;   // first slot of the odd harmonics in the paired layout
 constexpr int kTcMaxN = 256; // packed lengths the tensor-core path handles
 constexpr int kTcBN = 128;   // steered atoms per MMA (N) and per TMA box
-constexpr size_t kGramMax = (size_t)1 << 28;  // largest Gram table of the refine (bytes)
 constexpr int kTcMaxK = 8;   // greedy steps the tensor-core path handles
 
 constexpr int kTcSN = 256;   // steered atoms per chunk (MMA N) of the scoring pass
