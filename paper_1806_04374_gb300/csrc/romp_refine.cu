@@ -427,6 +427,32 @@ __global__ void __launch_bounds__(128, 4) romp_refine_kernel(const RefineArgs a)
         }
       }
     }
+    // a patch of zeros (a blank window) has nothing to code.  Its scores are all
+    // 0 and all inside the window: a small dictionary's were all re-scored, a
+    // large one's patch was handed off (100,000 blank patches at M = R = 16:
+    // 2.66 ms, 0.12 now; with a thread per patch it was 0.70)
+    if constexpr (T == 0) {
+      unsigned todo = __ballot_sync(0xffffffffu, act && xnorm == 0.0f);
+      while (todo) {
+        int src[B], slot;
+        next_batch<B>(todo, lane, src, slot);
+        unsigned some[B];
+#pragma unroll
+        for (int j = 0; j < B; ++j) {
+          float v[NS];
+          ls.load_x(a.x + (base + src[j]) * vec, v);
+          some[j] = 0;
+#pragma unroll
+          for (int u = 0; u < NS; ++u) some[j] |= v[u] != 0.0f;
+        }
+#pragma unroll
+        for (int j = 0; j < B; ++j)
+          if (!__any_sync(0xffffffffu, some[j]) && slot == j) {
+            outcome = 1;
+            qf = -1;
+          }
+      }
+    }
     auto umask_of = [&](int sl) {
       unsigned r = umk[0];
 #pragma unroll
