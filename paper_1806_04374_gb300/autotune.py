@@ -4,7 +4,10 @@ with CUDA events on a synthetic workload of the given sizes and writes the
 fastest per (n, M, R, K) to the table librsc reads when a dictionary is
 created (rsc_tuning.txt beside librsc.so; see include/rsc.h, "Tuning").
 
-A tuning never changes a result, so a candidate is judged on time alone.
+A tuning never changes a result, so a candidate is judged on time alone: the
+fastest call on device buffers, and among those within 1% of it the fastest call
+on host buffers, again to 1% (rsc_encode_host reads the same entry; its copies
+overlap best with other group counts than the kernels do).
 
 Usage (on the GPU):
     python -m paper_1806_04374_gb300.autotune [--workload NAME ...] [--out PATH]
@@ -76,6 +79,37 @@ def time_encode(dic, xd, K, reps: int) -> float:
     return float(np.median(ms))
 
 
+def time_encode_host(dic, x, K, reps: int) -> float:
+    """Milliseconds per rsc_encode_host (FP16 path) from and to pinned memory,
+    median of `reps` calls after one warm-up call."""
+    import torch
+    P = x.shape[0]
+    xh = torch.from_numpy(x).pin_memory()
+    out = {k: torch.empty((P, K) if k != "resid_norm2" else (P,), dtype=t, pin_memory=True)
+           for k, t in (("atom", torch.int32), ("angle_idx", torch.int32), ("angle", torch.float32),
+                        ("coef", torch.float64), ("resid_norm2", torch.float32))}
+    ms = []
+    for _ in range(reps + 1):
+        t0 = time.perf_counter()
+        rsc.encode_host(dic, xh, K, "f16", out=out)
+        ms.append(1e3 * (time.perf_counter() - t0))
+    return float(np.median(ms[1:]))
+
+
+def near_best(results) -> list[dict]:
+    """The candidates within 1% of the fastest call on device buffers."""
+    least = min(r["ms"] for r in results)
+    return [r for r in results if r["ms"] <= 1.01 * least]
+
+
+def pick(results) -> dict:
+    """The winner: of the candidates near the best, those within 1% of the
+    fastest call on host buffers; of these the fastest on device buffers."""
+    near = near_best(results)
+    least = min(r.get("host_ms", 0.0) for r in near)
+    return min((r for r in near if r.get("host_ms", 0.0) <= 1.01 * least), key=lambda r: r["ms"])
+
+
 def tune(name: str, reps: int = 3) -> dict:
     """Times every candidate on `name`'s sizes; returns the table entry of the
     fastest and every measurement."""
@@ -89,9 +123,13 @@ def tune(name: str, reps: int = 3) -> dict:
     for c in candidates(dic):
         rsc.rsc_dict_set_tuning(dic.handle, **c)
         results.append(dict(c, ms=time_encode(dic, xd, K, reps)))
+    for c in near_best(results):
+        rsc.rsc_dict_set_tuning(dic.handle, **{k: c[k] for k in
+                                               ("groups", "refine_blocks_per_sm", "score_stages")})
+        c["host_ms"] = time_encode_host(dic, x, K, reps)
     rsc.rsc_dict_set_tuning(dic.handle, clear=True)
     dic.close()
-    best = min(results, key=lambda r: r["ms"])
+    best = pick(results)
     n = J * (2 * kmax + 1)
     return {"workload": name, "n": n, "M": M, "R": R, "K": K, "patches": P,
             "best": best, "default_ms": next(r["ms"] for r in results
@@ -109,7 +147,8 @@ def table_lines(entries) -> list[str]:
         out.append(f"{e['n']} {e['M']} {e['R']} {e['K']} {b['groups']} 0 "
                    f"{b['refine_blocks_per_sm']} {b['score_stages']}"
                    f"  # {e['workload']}: {b['ms']:.3f} ms per call of {e['patches']} patches "
-                   f"(default {e['default_ms']:.3f} ms)")
+                   f"(default {e['default_ms']:.3f} ms)"
+                   + (f", {b['host_ms']:.3f} ms from host buffers" if "host_ms" in b else ""))
     return out
 
 
