@@ -80,7 +80,8 @@ typedef struct rsc_dict rsc_dict; /* opaque, device-resident, immutable */
  * proposed algorithm: atoms in steerable-basis coordinates) and precompute
  * its per-angle tables (the steering factors exp(-i k 2 pi r / R) of
  * Eq. (Sr), a transposed copy for the contraction, and, for the tensor-core
- * path, the steered dictionary S_r d_m in fp16, scaled by 256).
+ * path, the steered dictionary S_r d_m in fp16, scaled by 256, and again in
+ * double-float, and the inner products of the steered atoms).
  *   coef   : device pointer, M x (kmax+1) x J x 2 floats, atoms of unit
  *            norm (|<d,d> - 1| <= 1e-4, else RSC_ERR_INVALID); read once,
  *            the caller keeps ownership.
@@ -140,11 +141,12 @@ int rsc_encode(const rsc_dict *dict, const float *x, int64_t P, int32_t K, int32
  * For every atom m, each patch whose code uses m at angle r0 contributes the
  * column S_{-r0}(x_p - D_aug b_p), b_p = the patch's code without that (m, r0)
  * entry; the new atom is the first left singular vector of those columns,
- * computed as the leading eigenvector of their covariance (columns, products
- * and sums beyond FP32: C is off by some 1e-15 of its norm; FP64 power
- * iteration from the old atom, to convergence or 5000 iterations).  All atoms are updated from the dictionary `dict` and the same
- * codes.  Readings of the paper: a patch using m more than once contributes
- * its occurrence with the largest |weight| (ties: earliest); an atom used by
+ * computed as the leading eigenvector of their covariance (columns in
+ * double-float, products and sums beyond it: C is off by 1e-15 of its norm,
+ * by up to 1e-12 where residuals and weighted atoms cancel; FP64 power
+ * iteration from the old atom, to convergence or 5000 iterations).  All atoms
+ * are updated from the dictionary `dict` and the same codes.  Readings of the
+ * paper: a patch using m more than once contributes its occurrence with the largest |weight| (ties: earliest); an atom used by
  * no patch is reset to the unit-normalised patch with the largest coding
  * error (several: successive patches in descending error; at most 64
  * resets, further unused atoms keep their old value); the largest-magnitude

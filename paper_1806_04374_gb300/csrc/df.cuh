@@ -64,9 +64,6 @@ __device__ __forceinline__ df df_mul(df a, df b) {
   return fast_two_sum(p.hi, e);
 }
 
-// acc + a * b (a, b double-float).
-__device__ __forceinline__ df df_fma(df acc, df a, df b) { return df_add(acc, df_mul(a, b)); }
-
 __device__ __forceinline__ double df_to_d(df a) { return (double)a.hi + (double)a.lo; }
 
 __device__ __forceinline__ df df_from_d(double v) {

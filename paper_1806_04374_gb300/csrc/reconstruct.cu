@@ -274,9 +274,10 @@ cudaError_t launch_reconstruct(const rsc_dict *dict, int dev, int64_t P, int K, 
 // C[P][npix] = coef[P][nk] X[nk][npix], FP32 FMA in the order of the half
 // spectrum (the error of the plain sum; the tensor cores' accumulation is
 // coarser).  A block takes 16 RT rows and up to 128 pixels; thread (tx, ty)
-// of ct x 16 holds RT x 8 outputs.  Both operands stream through shared memory in chunks of kc coordinates with
-// cp.async, two chunks in flight.  ct, the threads across the pixels, is
-// chosen so that the last tile of pixels is full (97 pixels: 13 x 8 = 104).
+// of ct x 16 holds RT x 8 outputs.  Both operands stream through shared memory
+// in chunks of kc coordinates with cp.async, two chunks in flight.  ct, the
+// threads across the pixels, is chosen so that the last tile of pixels is full
+// (97 pixels: 13 x 8 = 104).
 // The result leaves through shared memory, so that its rows are written with
 // full lines.
 // 10^6 patches of 102 coordinates to 97 pixels: 0.68 ms (issue at 65%: seven

@@ -7,9 +7,9 @@
 //       lane per atom, FP32 FMA, the residual broadcast from shared memory;
 //   (b) angle transform score(m, r) = G_0 + 2 Re sum_k e^{ik 2 pi r / R} G_k,
 //       one lane per angle, or per pair of angles half a turn apart, with its
-//       cos/sin factors held in registers; with RSC_FP32_PRUNE only for the atoms whose exact bound |G_0| +
-//       2 sum_k |G_k| >= max_r |score(m, r)| can still reach the window of
-//       the running best;
+//       cos/sin factors held in registers; with RSC_FP32_PRUNE only for the
+//       atoms whose exact bound |G_0| + 2 sum_k |G_k| >= max_r |score(m, r)| can
+//       still reach the window of the running best;
 //   (c) per lane and angle the largest |score| and its runner-up, merged over
 //       the warp into every candidate within 2E of the best, where E bounds
 //       the FP32 error of a score; if a runner-up lies inside that window, the

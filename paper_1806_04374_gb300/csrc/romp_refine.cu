@@ -323,8 +323,8 @@ __global__ void __launch_bounds__(128) romp_init_kernel(const RefineArgs a) {
 // 0.98 at T = 1 / 2 / 3) against 1.06 for a thread per patch; the call 9.00 ->
 // 7.29 ms, 1,000 patches at M = 16 261 -> 129 us (one kernel per step, not a
 // memset and two passes; 81 with fewer patches a warp, see the launch), the
-// 21 x 21 image sizes 21.8 -> 16.3 ms.  Issue is at 50%, so both instructions (12,000 to 17,000 per warp) and the loads'
-// latency count.  Registers: at most 128 (4 blocks an SM) 3.79 ms per call of
+// 21 x 21 image sizes 21.8 -> 16.3 ms.  Issue is at 50%, so both instructions
+// (12,000 to 17,000 per warp) and the loads' latency count.  Registers: at most 128 (4 blocks an SM) 3.79 ms per call of
 // init and refines; without a cap (up to 255) 4.24, 5 or 6 blocks 3.96 / 3.91
 // (spills).
 template <int T, int LAY>

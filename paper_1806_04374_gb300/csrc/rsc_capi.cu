@@ -314,9 +314,11 @@ __global__ void anorm_kernel(const float *__restrict__ d, int M, int J, int H,
 }
 
 // Tables of the tensor-core path: the packed steered dictionary (fp16 of
-// kDictScale times the entries, row r*M + m = S_r d_m, angle-major so that 32 consecutive rows hold different
-// atoms; the packed layout described in rsc_internal.h), the
-// per-harmonic cross-Gram table H_k(a, b) in double-float and the TMA map.
+// kDictScale times the entries, row r*M + m = S_r d_m, angle-major so that 32
+// consecutive rows hold different atoms; the packed layout described in
+// rsc_internal.h), the refine's tables (dict_tables.h: the per-harmonic
+// cross-Gram H_k(a, b) in double-float, the norms, the steered rows in
+// double-float and the Gram entries) and the TMA map.
 // Returns RSC_OK also when the sizes are outside the path (tables left null).
 int build_tc_tables(rsc_dict *d, cudaStream_t st) {
   const int M = d->M, J = d->J, H = d->H, R = d->R;
@@ -549,8 +551,6 @@ int encode_f16_group(const rsc_dict *dict, const RompArgs &base, unsigned char *
   ra.kmax = dict->kmax;
   ra.R = dict->R;
   ra.H = dict->H;
-  ra.n = dict->n;
-  ra.d = dict->d;
   ra.tw = dict->tw;
   ra.xgram = dict->xgram;
   ra.anorm = dict->anorm;

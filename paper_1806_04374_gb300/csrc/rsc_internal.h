@@ -42,7 +42,8 @@ struct rsc_dict {
   // of the odd harmonics), else R; null when the allocator refused them
   float *rows;
   int Rr;
-  float2 *gram;          // [M][M][R] double-float <S_r d_a, d_b>; null when over kGramMax bytes or refused
+  float2 *gram;          // [M][M][R] double-float <S_r d_a, d_b>; null when over
+                         // kGramMax bytes (dict_tables.h) or refused
   int n;                 // packed real length J (2 kmax + 1)
   // per-phase timing (diagnostic): event pairs recorded around launches
   int timing;
@@ -232,8 +233,7 @@ int rsc_score_stage_options(int L, int paired, int *dflt, int *other);
 struct RefineArgs {
   const float *x;
   int64_t P;
-  int K, M, J, kmax, R, H, n;
-  const float *d;
+  int K, M, J, kmax, R, H;
   const float *tw;       // [4][H][R]
   const float4 *xgram;
   const float2 *anorm;   // [M] ||d_m||^2 in double-float
