@@ -47,3 +47,29 @@ def test_equal_columns(cuda_ok, P, scale):
             # slices are exact here, products kept down to 2^-53, the rest of
             # the sums (2^-30 of the whole) in FP32: 2^-49 with the last rounding
             assert abs(Fraction(float(C[i, j])) - ref) <= abs(ref) * Fraction(1, 2 ** 49), (i, j)
+
+
+@pytest.mark.parametrize("P", [1, 65, 321])
+def test_every_slice_counts(cuda_ok, P):
+    """Columns sqrt(2) x (weight 0, one angle): 48 bits each, cut into six
+    slices of 8.  A column is off by 2^-46 of itself (double-float: the product
+    with sqrt(2) 2^-47, its constant 2^-48) and its slices by 2^-48 of its row's
+    largest, so C by 2^-45 of the sum of moduli and 2^-47 of the products of the
+    largest; one slice left out shows 2^-42."""
+    import torch
+    import paper_1806_04374_gb300 as rsc
+    from oracle import ksvd
+    from paper_1806_04374_gb300 import synth
+    rsc.load_library()
+    J, kmax = 6, 8
+    x = np.random.default_rng(P).standard_normal((P, kmax + 1, J, 2)).astype(np.float32)
+    x[:, 0, :, 1] = 0.0
+    dic = rsc.Dictionary(torch.from_numpy(synth.make_dictionary(1, J, kmax, 3)).cuda(), 1)
+    zero = torch.zeros((P, 1), dtype=torch.int32, device="cuda")
+    C = rsc.ksvd_accumulate(dic, torch.from_numpy(x).cuda(), {
+        "atom": zero, "angle_idx": zero, "coef": zero.double()}, ntop=0)["C"][0].cpu().numpy()
+    dic.close()
+    y = ksvd.pack(x)
+    a, most = np.abs(y), np.abs(y).max(0)
+    tol = 2.0 ** -45 * (a.T @ a) + 2.0 ** -47 * P * np.outer(most, most)
+    assert np.all(np.abs(C - y.T @ y) <= tol)
