@@ -462,8 +462,8 @@ __global__ void __launch_bounds__(kCovThreads) ksvd_cov_kernel(const KsvdArgs a)
 //   * warp 23 (one lane) issues the MMAs (M = 128, N = n padded to 16).
 // Rows hold the real parts of the entries first, then the imaginary parts of
 // k >= 1, so that neighbouring lanes store to neighbouring rows.
-// 200,000 patches, K = 5, M = 128, n = 102, R = 64 (10^6 samples): 1.07 ms, and
-// the whole accumulation and update 1.63 ms (6.86 ms with every covariance on
+// 200,000 patches, K = 5, M = 128, n = 102, R = 64 (10^6 samples): 1.06 ms, and
+// the whole accumulation and update 1.60 ms (6.86 ms with every covariance on
 // the CUDA cores); C off by 1.8e-15 of its norm, 1.9e-15 there.
 // Every wait is bounded.  One that runs out is reported twice: in the
 // dictionary's error word, and as a slice without a sum (kCvFailed), which

@@ -47,14 +47,14 @@ __device__ __forceinline__ float2 halves(f32x2 v) {
 // entries of one patch's harmonic: it forms the steered weights
 // a_i e^{-i k theta_i} in double-float once per term and applies them to its
 // entries' FP32 atoms, accumulating to about 60 bits.
-// 10^6 patches of 54 entries, K = 5: 0.53 ms (the operations themselves 0.21
+// 10^6 patches of 54 entries, K = 5: 0.52 ms (the operations themselves 0.21
 // at the FP32 peak; a two-element FMA takes 2.3 cycles, so it saves issue
 // slots and no time on the pipe), against 7.0 ms for FP64 throughout (15
 // operations per term on a pipe of 1/64 of the FP32 rate, every factor formed
 // again for every entry); the memory floor is 75 us.  With two floats for an
 // accumulator (48 bits, 0.42 ms) entries that cancel to 2^-20 of the weights
 // came out up to 7 x 2^-24 off.  Four entries a lane 0.73 ms, a third block an
-// SM (80 registers, spills) 0.55; of the time 5% are the entries in FP64.
+// SM (80 registers, spills) 0.54; of the time 5% are the entries in FP64.
 constexpr int kRecThreads = 256;
 constexpr int kRecTile = 32;   // patches per warp and tile
 constexpr int kRecEntries = 6;

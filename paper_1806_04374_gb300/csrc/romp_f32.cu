@@ -28,7 +28,7 @@
 // a patch and step at M = 64, R = 64, K = 5; the code's traffic is the input
 // once).  With a branching top-4 insert for every value, no pairs and the
 // factor on lane 0 it took 10.5 thousand at 59%: 100,003 patches 7.42 ms then,
-// 3.14 ms now.  The exact part's loops are kept rolled: unrolled, their code
+// 3.15 ms now.  The exact part's loops are kept rolled: unrolled, their code
 // overran the instruction cache (4.24 against 3.58 ms).
 #include <math.h>
 
