@@ -249,8 +249,10 @@ __global__ void __launch_bounds__((32 * BlockWarps<KM, RPL, PRUNE>::v))
   // The branch-free pass over the scores is tried first unless this warp's
   // last step had a runner-up in the window: dictionaries with coinciding
   // atoms have one at every step, and the pass would only come on top (50,000
-  // patches, M = 64 in pairs, K = 5: 4.15 ms with it at R = 33 and 2.78 without,
-  // 3.34 and 2.35 at R = 64).
+  // patches, M = 64 in pairs, K = 5: 4.15 ms with it at R = 33 and 2.77 without,
+  // 3.34 and 2.35 at R = 64).  Not so for patches that the FP16 path hands over:
+  // they begin with such a step, and it says little of the next (25 us of the
+  // 3.9 ms of 350,000 11 x 11 windows).
   bool fast = !PRUNE;
   for (int64_t it = (int64_t)blockIdx.x * warps + warp;; it += nwarps) {
     int64_t p;
@@ -457,8 +459,11 @@ __global__ void __launch_bounds__((32 * BlockWarps<KM, RPL, PRUNE>::v))
           } else {
             close = tv[1] >= thr;
           }
-          if constexpr (!PRUNE) fast = !__any_sync(0xffffffffu, close);
-          if (!first || fast) break;
+          if constexpr (!PRUNE) {
+            close = __any_sync(0xffffffffu, close);
+            fast = a.redo_list || !close;
+          }
+          if (!first || !close) break;
           first = false;
         }
         if (done) break;
